@@ -67,7 +67,12 @@ enum {
 enum { ECC_F32 = 0, ECC_F16 = 1, ECC_BF16 = 2 };
 
 /* Device status bits returned by ecc_status() (and in ecc_result.flags). */
-enum { ECC_STATUS_DEGENERATE_VIEW = 1, ECC_STATUS_DEGENERATE_PAIR = 2, ECC_STATUS_NONFINITE_PAIR = 4 };
+enum {
+  ECC_STATUS_DEGENERATE_VIEW = 1,
+  ECC_STATUS_DEGENERATE_PAIR = 2,
+  ECC_STATUS_NONFINITE_PAIR = 4,
+  ECC_STATUS_TIMEOUT = 8 /* a bounded device wait of a precompute gave up: its sinograms are not valid */
+};
 
 /* Library version (major * 10000 + minor * 100 + patch). */
 int ecc_version(void);

@@ -162,38 +162,43 @@ int check_geometry_args(ecc_ctx* c, int n_views, const void* P, int W, int H, in
 }
 
 
-// Views per dRadon/ds batch: the weighted images of a batch take at most 256 MiB.
-int radon_batch_views(int n_views, int W, int H, int n_s) {
-  const size_t plane = ecc::radon_plane_bytes(W, H, n_s);
-  const size_t max_batch_bytes = (size_t)256 << 20;
-  return (int)std::max<size_t>(1, std::min<size_t>((size_t)n_views, max_batch_bytes / plane));
-}
+// Scratch of the many-view precompute: enough for ten groups of 32 views on a 620 x 480
+// detector, or for four on a 976 x 976 one.
+constexpr size_t kViewsScratch = (size_t)1152 << 20;
+constexpr int kHostBatch = 128;  // views per upload of the host-buffer call
 
-// batch_ready (or NULL): one event per batch, which the stream waits for before the
-// batch reads its images.
-int run_precompute(ecc_ctx* c, int n_views, const double* P, const float* images, int W, int H, int n_alpha, int n_s,
-                   int dtype, void* sino_out, float* scales_out, cudaStream_t s,
-                   const cudaEvent_t* batch_ready = nullptr) {
+// Scratch of a precompute and the plan that fits it: the many-view form on less and less
+// scratch, at last view by view, within the context's budget.
+int ensure_precompute(ecc_ctx* c, int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
+                      ecc::RadonPlan* plan) {
   int rc;
   if ((rc = ensure(c, c->views, sizeof(ecc::ViewRec) * (size_t)n_views, "views")) != ECC_OK) return rc;
-  const size_t tbytes = sizeof(ecc::RadonRow) * (size_t)n_views * n_alpha + sizeof(ecc::RadonView) * (size_t)n_views;
-  if ((rc = ensure(c, c->rtable, tbytes, "radon table")) != ECC_OK) return rc;
-  const size_t plane = ecc::radon_plane_bytes(W, H, n_s);
-  const int batch = radon_batch_views(n_views, W, H, n_s);
-  if ((rc = ensure(c, c->wimg, plane * (size_t)batch, "weighted images")) != ECC_OK) return rc;
-  if (dtype == ECC_F16 &&
-      (rc = ensure(c, c->stage, ecc::radon_f16_stage_bytes(n_alpha, n_s, batch), "FP16 staging")) != ECC_OK)
-    return rc;
+  size_t cap = kViewsScratch;
+  for (;;) {
+    *plan = ecc::radon_plan(n_views, W, H, n_alpha, n_s, dtype, max_batch, cap, 0);
+    rc = ensure(c, c->rtable, plan->table_bytes(n_views, n_alpha), "radon table");
+    if (rc == ECC_OK) rc = ensure(c, c->wimg, plan->wimg_bytes, "weighted images");
+    if (rc == ECC_OK && plan->stage_bytes) rc = ensure(c, c->stage, plan->stage_bytes, "FP16 staging");
+    if (rc == ECC_OK || !plan->views) return rc;
+    cap = plan->batch > 32 ? plan->wimg_bytes / 2 : plan->wimg_bytes - 1;
+  }
+}
+
+// batch_ready (or NULL): one event per batch of the plan, which the stream waits for
+// before the batch reads its images.
+int run_precompute(ecc_ctx* c, int n_views, const double* P, const float* images, int W, int H, int n_alpha, int n_s,
+                   int dtype, void* sino_out, float* scales_out, const ecc::RadonPlan& plan, cudaStream_t s,
+                   const cudaEvent_t* batch_ready = nullptr) {
+  cudaError_t e;
   const ecc::LaunchHooks hk = hooks_of(c);
   hk.on_begin("view_setup_kernel", s);
   ecc::view_setup_kernel<<<(n_views + 127) / 128, 128, 0, s>>>(n_views, P, nullptr, W, H, (ecc::ViewRec*)c->views.p,
                                                               c->d_status);
   hk.on_end("view_setup_kernel", s);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(c, e, "view set-up launch");
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "view set-up launch");
   e = ecc::launch_radon((const ecc::ViewRec*)c->views.p, n_views, images, W, H, n_alpha, n_s, dtype, sino_out,
-                        scales_out, (ecc::RadonRow*)c->rtable.p, c->wimg.p, (float*)c->stage.p, batch, hk, s,
-                        batch_ready);
+                        scales_out, (ecc::RadonRow*)c->rtable.p, c->wimg.p, (float*)c->stage.p, plan, c->d_status, hk,
+                        s, batch_ready);
   if (e != cudaSuccess) return cuda_fail(c, e, "radon launch");
   return ECC_OK;
 }
@@ -441,7 +446,9 @@ int ecc_precompute_radon_derivative(ecc_ctx* c, int n_views, const double* P, co
   if (!images || !sino_out) return fail(c, ECC_EINVAL, "images or sino_out is NULL");
   if (dtype == ECC_F16 && !scales_out) return fail(c, ECC_EINVAL, "ECC_F16 needs scales_out");
   DeviceGuard g(c->device);
-  return run_precompute(c, n_views, P, images, W, H, n_alpha, n_s, dtype, sino_out, scales_out,
+  ecc::RadonPlan plan;
+  if ((rc = ensure_precompute(c, n_views, W, H, n_alpha, n_s, dtype, n_views, &plan)) != ECC_OK) return rc;
+  return run_precompute(c, n_views, P, images, W, H, n_alpha, n_s, dtype, sino_out, scales_out, plan,
                         (cudaStream_t)stream);
 }
 
@@ -540,7 +547,9 @@ int ecc_scan_consistency_host(ecc_ctx* c, int n_views, const double* P_host, con
   // From pinned host memory the images go up per precompute batch on a second stream,
   // so that the upload of batch b + 1 overlaps the projection of batch b; pageable
   // memory (whose asynchronous copies block the host) is copied in one piece.
-  const int batch = radon_batch_views(n_views, W, H, n_s);
+  ecc::RadonPlan plan;
+  if ((rc = ensure_precompute(c, n_views, W, H, n_alpha, n_s, ECC_F32, kHostBatch, &plan)) != ECC_OK) return rc;
+  const int batch = plan.batch;
   const int n_batches = (n_views + batch - 1) / batch;
   cudaPointerAttributes pa;
   const bool pinned = cudaPointerGetAttributes(&pa, images_host) == cudaSuccess && pa.type == cudaMemoryTypeHost;
@@ -575,7 +584,7 @@ int ecc_scan_consistency_host(ecc_ctx* c, int n_views, const double* P_host, con
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "host-to-device copy");
   rc = run_precompute(c, n_views, (const double*)c->h_P.p, (const float*)c->h_img.p, W, H, n_alpha, n_s, ECC_F32,
-                      c->h_sino.p, nullptr, s, ready.ev.empty() ? nullptr : ready.ev.data());
+                      c->h_sino.p, nullptr, plan, s, ready.ev.empty() ? nullptr : ready.ev.data());
   if (rc != ECC_OK) return rc;
   rc = run_evaluate(c, n_views, (const double*)c->h_P.p, nullptr, c->h_sino.p, nullptr, W, H, n_alpha, n_s, ECC_F32,
                     n_kappa, cauchy_c, nullptr, (int)np, (double*)c->h_total.p, nullptr, nullptr, nullptr, nullptr, false,

@@ -59,6 +59,7 @@ enum : int {
   kStatusDegenerateView = 1,
   kStatusDegeneratePair = 2,
   kStatusNonfinitePair = 4,  // a pair's sum (or its gradient) was not finite: zeroed
+  kStatusTimeout = 8,        // a bounded device wait gave up: the call's sinograms are not valid
 };
 
 // A unit direction (x, y) split into double-float pairs: (hi.x, hi.y, lo.x, lo.y).

@@ -2,6 +2,7 @@
 #pragma once
 #include <cmath>
 #include <cstdint>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include "ecc_internal.cuh"
 
@@ -24,7 +25,7 @@ __global__ void view_grad_P_kernel(int n_views, long long n_pairs, const int32_t
                                    const ViewTanP* vtan, double* grad_P);
 __global__ void alpha_dir_kernel(int n_alpha, float4* dir);
 
-// Per (view, alpha-row) line parameters of the Joseph line sums (32.32 fixed point).
+// Line parameters of the Joseph line sums at one alpha row (32.32 fixed point).
 struct RadonRow {
   long long B0;    // coordinate along the interpolation axis at rho index 0, step 0
   long long STEP;  // per rho index
@@ -88,15 +89,40 @@ inline void pair_args_grid(PairArgs& g, int n_alpha, int n_s, int W, int H) {
   g.half_lo = (float)(half - (double)g.half_hi);
 }
 
+// How a dRadon/ds precompute runs, by its sizes and the scratch it may use.  Scans with
+// enough views whose grid qualifies follow the detector lines once for many views
+// (radon_views.cu), others view by view (radon.cu).  The choice between the two
+// depends on the sizes alone, and the many-view sums do not depend on how the views are
+// grouped, so that a scan's sinograms are the same wherever they are computed.
+struct RadonPlan {
+  bool views;          // many views at once
+  int batch;           // views per pass over the scratch
+  size_t wimg_bytes;   // weighted images
+  size_t stage_bytes;  // FP32 staging of FP16 storage
+  size_t table_bytes(int n_views, int n_alpha) const;  // line table and per-view weights
+};
+// At most max_batch views per pass; wimg_cap bounds the many-view form's scratch and
+// total_cap (0: none) its scratch and staging together.  Where no group of views fits
+// the plan is the view-by-view form's.
+RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch, size_t wimg_cap,
+                     size_t total_cap);
+
+// Many-view form, in groups of 32 views.
+struct ViewsPlan {
+  // least number of views for which the many-view form is taken; 0: the grid does not qualify
+  static int min_views(int W, int H, int n_alpha, int n_s);
+  // scratch of one group with the planes of both axes (2) or of one at a time (1)
+  static size_t group_bytes(int axes, int W, int H, int n_alpha, int n_s);
+};
+
 // Launchers (return cudaError_t of the launch).
 cudaError_t launch_radon(const ViewRec* views, int n_views, const float* images, int W, int H, int n_alpha, int n_s,
                          int dtype, void* sino_out, float* scales_out, RadonRow* table, void* wimg, float* stage,
-                         int batch_views, const LaunchHooks& hooks, cudaStream_t stream,
+                         const RadonPlan& plan, int* status, const LaunchHooks& hooks, cudaStream_t stream,
                          const cudaEvent_t* batch_ready = nullptr);  // per batch: wait before reading its images
-size_t radon_f16_stage_bytes(int n_alpha, int n_s, int batch_views);
-int radon_pad(int W, int H, int n_s);
-// Bytes of one view's weighted-image planes (interpolation pairs, both orientations).
-size_t radon_plane_bytes(int W, int H, int n_s);
+cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n_views, const float* images, int W,
+                               int H, int n_alpha, int n_s, void* planes, size_t plane_bytes, float* of,
+                               __nv_bfloat16* ob, int* status, const LaunchHooks& hooks, cudaStream_t stream);
 
 cudaError_t launch_ecc_pairs(long long n_pairs, const PairRec* prs, const float4* ctile, int n_tiles,
                              const float4* alpha_dir, const void* sino, const float* scales, int dtype,

@@ -1,7 +1,7 @@
 // dRadon/ds precompute: the Grangeat intermediate function S_lambda (Eq. 1) of
 // every projection on an (alpha, s) grid.
 //
-//   radon_table_kernel   FP64, one thread per (view, alpha row): the parameters of
+//   radon_table_kernel   FP64, one thread per alpha row (and view): the parameters of
 //                        the detector lines (x - cx) cos a + (y - cy) sin a = sigma
 //                        as 32.32 fixed-point coordinates along the interpolation
 //                        axis (exact integer stepping, no FP64 in the hot loop).
@@ -33,11 +33,24 @@ namespace {
 
 constexpr double kTwo32 = 4294967296.0;
 
-__global__ void radon_table_kernel(const ViewRec* __restrict__ views, int n_views, int W, int H, int n_alpha,
-                                   int n_s, RadonRow* __restrict__ table, RadonView* __restrict__ rv) {
+// copies: the line parameters are the same for every view; the view-by-view form reads a
+// copy per view (its kernel, indexed so, compiles to 64 registers and four blocks per SM;
+// with one shared copy it takes 48, and the bands of five blocks thrash L1: 65 us against
+// 31 on two 256 x 256 views), the many-view form one.
+__global__ void radon_table_kernel(const ViewRec* __restrict__ views, int n_views, int copies, int W, int H,
+                                   int n_alpha, int n_s, RadonRow* __restrict__ table,
+                                   RadonView* __restrict__ rv) {
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)n_views * n_alpha) return;
-  const int v = (int)(idx / n_alpha);
+  if (idx < n_views) {
+    const ViewRec& vr = views[idx];
+    RadonView o;
+    o.u0 = (float)vr.u0;
+    o.v0 = (float)vr.v0;
+    o.D = (float)vr.D;
+    o.pad = 0;
+    rv[idx] = o;
+  }
+  if (idx >= (long long)copies * n_alpha) return;
   const int m = (int)(idx % n_alpha);
   double sa, ca;
   sincospi((double)m / (double)n_alpha, &sa, &ca);
@@ -65,15 +78,6 @@ __global__ void radon_table_kernel(const ViewRec* __restrict__ views, int n_view
   r.sa = (float)sa;
   r.rows_mode = rows ? 1 : 0;
   table[idx] = r;
-  if (m == 0) {
-    const ViewRec& vr = views[v];
-    RadonView o;
-    o.u0 = (float)vr.u0;
-    o.v0 = (float)vr.v0;
-    o.D = (float)vr.D;
-    o.pad = 0;
-    rv[v] = o;
-  }
 }
 
 // Weighted projection as interpolation pairs (v[i], v[i+1] - v[i]) along the
@@ -302,17 +306,68 @@ size_t radon_f16_stage_bytes(int n_alpha, int n_s, int batch_views) {
   return sizeof(float) * (size_t)n_alpha * n_s * batch_views;
 }
 
+size_t RadonPlan::table_bytes(int n_views, int n_alpha) const {
+  return sizeof(RadonRow) * (size_t)(views ? 1 : n_views) * n_alpha + sizeof(RadonView) * (size_t)n_views;
+}
+
+RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch, size_t wimg_cap,
+                     size_t total_cap) {
+  RadonPlan p{};
+  auto stage = [&](int batch) { return dtype == 1 ? radon_f16_stage_bytes(n_alpha, n_s, batch) : (size_t)0; };
+  const int least = ViewsPlan::min_views(W, H, n_alpha, n_s);
+  if (least > 0 && n_views >= least) {
+    for (int axes = 2; axes >= 1; --axes) {
+      const size_t gb = ViewsPlan::group_bytes(axes, W, H, n_alpha, n_s);
+      int groups = (int)std::min<size_t>((size_t)(n_views + 31) / 32, wimg_cap / gb);
+      groups = std::min(groups, (max_batch + 31) / 32);
+      auto batch = [&] { return std::min(n_views, groups * 32); };
+      while (groups > 0 && total_cap && gb * groups + stage(batch()) > total_cap) --groups;
+      if (groups == 0) continue;
+      p.views = true;
+      p.batch = batch();
+      p.wimg_bytes = gb * groups;
+      p.stage_bytes = stage(p.batch);
+      return p;
+    }
+  }
+  const size_t plane = radon_plane_bytes(W, H, n_s);
+  const size_t max_batch_bytes = (size_t)256 << 20;  // weighted images of a batch, unless one view takes more
+  p.batch = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_views, max_batch_bytes / plane));
+  p.wimg_bytes = plane * (size_t)p.batch;
+  p.stage_bytes = stage(p.batch);
+  return p;
+}
+
+// FP16 storage of nb views staged in FP32: per-view maximum, scale, quantisation.
+static cudaError_t quantize_batch(const float* stage, size_t per_view, int nb, float* scales, __half* out,
+                                  const LaunchHooks& hooks, cudaStream_t stream) {
+  const cudaError_t e = cudaMemsetAsync(scales, 0, sizeof(float) * nb, stream);
+  if (e != cudaSuccess) return e;
+  const unsigned per_block = 256 * 16;  // 16 elements per thread, at most 64 blocks per view
+  const unsigned bpv = (unsigned)std::min<size_t>(64, (per_view + per_block - 1) / per_block);
+  hooks.on_begin("absmax_kernel", stream);
+  absmax_kernel<<<dim3(bpv, nb), 256, 0, stream>>>(stage, per_view, reinterpret_cast<unsigned*>(scales));
+  hooks.on_end("absmax_kernel", stream);
+  scale_finalize_kernel<<<(nb + 255) / 256, 256, 0, stream>>>(scales, nb);
+  const size_t n = per_view * nb;
+  hooks.on_begin("quantize_f16_kernel", stream);
+  quantize_f16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(stage, per_view, n, scales, out);
+  hooks.on_end("quantize_f16_kernel", stream);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_radon(const ViewRec* views, int n_views, const float* images, int W, int H, int n_alpha, int n_s,
                          int dtype, void* sino_out, float* scales_out, RadonRow* table, void* wimg,
-                         float* stage, int batch_views, const LaunchHooks& hooks, cudaStream_t stream,
-                         const cudaEvent_t* batch_ready) {
+                         float* stage, const RadonPlan& plan, int* status, const LaunchHooks& hooks,
+                         cudaStream_t stream, const cudaEvent_t* batch_ready) {
   // table and per-view weights (RadonView array sits right after the table)
-  RadonView* rv = reinterpret_cast<RadonView*>(table + (size_t)n_views * n_alpha);
+  const int copies = plan.views ? 1 : n_views;
+  RadonView* rv = reinterpret_cast<RadonView*>(table + (size_t)copies * n_alpha);
   {
-    const long long n = (long long)n_views * n_alpha;
+    const long long n = std::max((long long)n_views, (long long)copies * n_alpha);
     hooks.on_begin("radon_table_kernel", stream);
-    radon_table_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(views, n_views, W, H, n_alpha, n_s, table,
-                                                                       rv);
+    radon_table_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(views, n_views, copies, W, H, n_alpha, n_s,
+                                                                       table, rv);
     hooks.on_end("radon_table_kernel", stream);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -329,50 +384,44 @@ cudaError_t launch_radon(const ViewRec* views, int n_views, const float* images,
   jg.plane = radon_plane_bytes(W, H, n_s) / sizeof(float2);
   jg.ds = (float)(sqrt((double)W * W + (double)H * H) / (n_s - 1));
   const int n_chunks = (n_s + 30) / 31;
+  const size_t per_view = (size_t)n_alpha * n_s;
   float2* wv = reinterpret_cast<float2*>(wimg);
-  for (int v0 = 0; v0 < n_views; v0 += batch_views) {
-    const int nb = min(batch_views, n_views - v0);
+  for (int v0 = 0; v0 < n_views; v0 += plan.batch) {
+    const int nb = min(plan.batch, n_views - v0);
     cudaError_t e;
-    if (v0 == 0) {  // zero margins; later batches overwrite only the pairs of the image
-      e = cudaMemsetAsync(wimg, 0, sizeof(float2) * jg.plane * nb, stream);
-      if (e != cudaSuccess) return e;
-    }
-    if (batch_ready && (e = cudaStreamWaitEvent(stream, batch_ready[v0 / batch_views], 0)) != cudaSuccess) return e;
-    hooks.on_begin("weight_kernel", stream);
-    weight_kernel<<<dim3((W + 32) / 32, (H + 32) / 32, nb), dim3(32, 8), 0, stream>>>(
-        images + (size_t)v0 * W * H, rv + v0, W, H, jg.pad, jg.pitch_r, jg.pitch_c, wv, jg.plane);
-    hooks.on_end("weight_kernel", stream);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const RadonRow* tb = table + (size_t)v0 * n_alpha;
-    const size_t oo = (size_t)v0 * n_alpha * n_s;
+    if (batch_ready && (e = cudaStreamWaitEvent(stream, batch_ready[v0 / plan.batch], 0)) != cudaSuccess) return e;
+    const float* im = images + (size_t)v0 * W * H;
+    const size_t oo = (size_t)v0 * per_view;
     float* of = dtype == 0 ? (float*)sino_out + oo : (dtype == 1 ? stage : nullptr);
     __nv_bfloat16* ob = dtype == 2 ? (__nv_bfloat16*)sino_out + oo : nullptr;
-    const dim3 grid(n_chunks, (n_alpha + kAlphaPerBlock - 1) / kAlphaPerBlock, nb), block(32 * kAlphaPerBlock);
-    hooks.on_begin("joseph_kernel", stream);
-    if (clamp)
-      joseph_kernel<true><<<grid, block, 0, stream>>>(tb, rv + v0, wv, jg, of, ob);
-    else
-      joseph_kernel<false><<<grid, block, 0, stream>>>(tb, rv + v0, wv, jg, of, ob);
-    hooks.on_end("joseph_kernel", stream);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (dtype == 1) {
-      const size_t per_view = (size_t)n_alpha * n_s;
-      e = cudaMemsetAsync(scales_out + v0, 0, sizeof(float) * nb, stream);
+    if (plan.views) {
+      e = launch_radon_views(table, rv + v0, nb, im, W, H, n_alpha, n_s, wimg, plan.wimg_bytes, of, ob, status, hooks,
+                             stream);
       if (e != cudaSuccess) return e;
-      const unsigned per_block = 256 * 16;  // 16 elements per thread, at most 64 blocks per view
-      const unsigned bpv = (unsigned)std::min<size_t>(64, (per_view + per_block - 1) / per_block);
-      hooks.on_begin("absmax_kernel", stream);
-      absmax_kernel<<<dim3(bpv, nb), 256, 0, stream>>>(stage, per_view, reinterpret_cast<unsigned*>(scales_out + v0));
-      hooks.on_end("absmax_kernel", stream);
-      scale_finalize_kernel<<<(nb + 255) / 256, 256, 0, stream>>>(scales_out + v0, nb);
-      const size_t n = per_view * nb;
-      hooks.on_begin("quantize_f16_kernel", stream);
-      quantize_f16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(
-          stage, per_view, n, scales_out + v0, (__half*)sino_out + (size_t)v0 * per_view);
-      hooks.on_end("quantize_f16_kernel", stream);
+    } else {
+      if (v0 == 0) {  // zero margins; later batches overwrite only the pairs of the image
+        e = cudaMemsetAsync(wimg, 0, sizeof(float2) * jg.plane * nb, stream);
+        if (e != cudaSuccess) return e;
+      }
+      hooks.on_begin("weight_kernel", stream);
+      weight_kernel<<<dim3((W + 32) / 32, (H + 32) / 32, nb), dim3(32, 8), 0, stream>>>(
+          im, rv + v0, W, H, jg.pad, jg.pitch_r, jg.pitch_c, wv, jg.plane);
+      hooks.on_end("weight_kernel", stream);
       e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+      const RadonRow* tb = table + (size_t)v0 * n_alpha;
+      const dim3 grid(n_chunks, (n_alpha + kAlphaPerBlock - 1) / kAlphaPerBlock, nb), block(32 * kAlphaPerBlock);
+      hooks.on_begin("joseph_kernel", stream);
+      if (clamp)
+        joseph_kernel<true><<<grid, block, 0, stream>>>(tb, rv + v0, wv, jg, of, ob);
+      else
+        joseph_kernel<false><<<grid, block, 0, stream>>>(tb, rv + v0, wv, jg, of, ob);
+      hooks.on_end("joseph_kernel", stream);
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
+    if (dtype == 1) {
+      e = quantize_batch(stage, per_view, nb, scales_out + v0, (__half*)sino_out + oo, hooks, stream);
       if (e != cudaSuccess) return e;
     }
   }

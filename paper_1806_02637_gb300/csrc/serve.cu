@@ -55,7 +55,7 @@ struct Layout {  // byte offsets of a job's resident and transient sections
   size_t P, theta, grad, views, vtan, adir, sino, scales, prs, ctile, partial, Gpp, gpp, totals, status;
   size_t theta0, nodes, jac, jbase, resident;
   size_t images, rtable, wimg, stage, transient;
-  int batch;
+  ecc::RadonPlan plan;
 };
 
 Layout layout_of(const ecc_job& j) {
@@ -92,11 +92,20 @@ Layout layout_of(const ecc_job& j) {
   L.resident = o;
   o = 0;
   L.images = take(n * (size_t)j.W * j.H * sizeof(float));
-  L.rtable = take(n * (size_t)j.n_alpha * sizeof(ecc::RadonRow) + n * sizeof(ecc::RadonView));
-  const size_t plane = ecc::radon_plane_bytes(j.W, j.H, j.n_s);
-  L.batch = (int)std::max<size_t>(1, std::min<size_t>(n, ((size_t)256 << 20) / plane));
-  L.wimg = take(plane * (size_t)L.batch);
-  L.stage = take(j.dtype == ECC_F16 ? ecc::radon_f16_stage_bytes(j.n_alpha, j.n_s, L.batch) : 0);
+  // The precompute's scratch is that of the view-by-view form, in which the many-view
+  // form takes the largest groups that fit: a job's footprint does not depend on the form.
+  const ecc::RadonPlan by_view = ecc::radon_plan((int)n, j.W, j.H, j.n_alpha, j.n_s, j.dtype, (int)n, 0, 0);
+  L.rtable = take(by_view.table_bytes((int)n, j.n_alpha));
+  L.wimg = take(by_view.wimg_bytes);
+  L.stage = take(by_view.stage_bytes);
+  L.plan.views = true;
+  const size_t wimg = align256(L.rtable + L.plan.table_bytes((int)n, j.n_alpha));
+  const size_t room = o - wimg - 256;
+  L.plan = ecc::radon_plan((int)n, j.W, j.H, j.n_alpha, j.n_s, j.dtype, (int)n, room, room);
+  if (L.plan.views) {
+    L.wimg = wimg;
+    L.stage = wimg + align256(L.plan.wimg_bytes);
+  }
   L.transient = o;
   return L;
 }
@@ -217,7 +226,8 @@ bool admit_job(ecc_serve* S, Job* J) {
     const ecc::LaunchHooks hk;
     e = ecc::launch_radon((const ecc::ViewRec*)(R + L.views), (int)n, (const float*)(T + L.images), d.W, d.H,
                           d.n_alpha, d.n_s, d.dtype, R + L.sino, (float*)(R + L.scales),
-                          (ecc::RadonRow*)(T + L.rtable), T + L.wimg, (float*)(T + L.stage), L.batch, hk, s);
+                          (ecc::RadonRow*)(T + L.rtable), T + L.wimg, (float*)(T + L.stage), L.plan,
+                          (int*)(R + L.status), hk, s);
   }
   if (e != cudaSuccess) {
     set_err(J, ECC_ECUDA, cuda_msg("precompute launch", e));
