@@ -796,7 +796,7 @@ def run_ours(args):
                 "frac": achieved / peak, "traffic": None,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if "hbm_gbs" in peaks else "fallback",
                 "work": "32 B (2 views x 4 taps x FP32) per line-pair sample"}
-    ev_names = ("view_setup_kernel", "alpha_dir_kernel", "pair_setup_kernel", "ecc_pair_kernel", "reduce_kernel")
+    ev_names = ("geometry_kernel", "pair_setup_kernel", "ecc_pair_kernel", "reduce_kernel")
     eval_ms = wall_ms(lambda: ecc.ecc_evaluate(ctx, P, sino, cfg.W, cfg.H, cfg.K, total=total, want_per_pair=False),
                       10)
     pk = kern.get("ecc_pair_kernel")

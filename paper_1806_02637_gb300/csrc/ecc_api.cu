@@ -191,14 +191,22 @@ int run_precompute(ecc_ctx* c, int n_views, const double* P, const float* images
                    const cudaEvent_t* batch_ready = nullptr) {
   cudaError_t e;
   const ecc::LaunchHooks hk = hooks_of(c);
-  hk.on_begin("view_setup_kernel", s);
-  ecc::view_setup_kernel<<<(n_views + 127) / 128, 128, 0, s>>>(n_views, P, nullptr, W, H, (ecc::ViewRec*)c->views.p,
-                                                              c->d_status);
-  hk.on_end("view_setup_kernel", s);
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "view set-up launch");
-  e = ecc::launch_radon((const ecc::ViewRec*)c->views.p, n_views, images, W, H, n_alpha, n_s, dtype, sino_out,
-                        scales_out, (ecc::RadonRow*)c->rtable.p, c->wimg.p, (float*)c->stage.p, plan, c->d_status, hk,
-                        s, batch_ready);
+  ecc::RadonRow* table = (ecc::RadonRow*)c->rtable.p;
+  ecc::Geometry g{};
+  g.n_views = n_views;
+  g.W = W;
+  g.H = H;
+  g.P = P;
+  g.views = (ecc::ViewRec*)c->views.p;
+  g.status = c->d_status;
+  g.weights = plan.weights(table, n_views, n_alpha);
+  g.n_alpha = n_alpha;
+  g.n_s = n_s;
+  g.table = table;
+  g.copies = plan.copies(n_views);
+  if ((e = ecc::launch_geometry(g, hk, s)) != cudaSuccess) return cuda_fail(c, e, "geometry launch");
+  e = ecc::launch_radon(n_views, images, W, H, n_alpha, n_s, dtype, sino_out, scales_out, table, c->wimg.p,
+                        (float*)c->stage.p, plan, c->d_status, hk, s, batch_ready);
   if (e != cudaSuccess) return cuda_fail(c, e, "radon launch");
   return ECC_OK;
 }
@@ -250,19 +258,22 @@ int run_evaluate(ecc_ctx* c, int n_views, const double* P, const double* motion,
   }
   if (!reuse) c->samp_valid = false;
   const ecc::LaunchHooks hk = hooks_of(c);
-  hk.on_begin("view_setup_kernel", s);
-  ecc::view_setup_kernel<<<(n_views + 127) / 128, 128, 0, s>>>(n_views, P, motion, W, H, (ecc::ViewRec*)c->views.p,
-                                                              c->d_status);
-  hk.on_end("view_setup_kernel", s);
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "view set-up launch");
-  if (c->adir_n != n_alpha || c->adir_ptr != c->adir.p) {  // the table depends on n_alpha only
-    hk.on_begin("alpha_dir_kernel", s);
-    ecc::alpha_dir_kernel<<<(n_alpha + 255) / 256, 256, 0, s>>>(n_alpha, (float4*)c->adir.p);
-    hk.on_end("alpha_dir_kernel", s);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "alpha table launch");
-    c->adir_n = n_alpha;
-    c->adir_ptr = c->adir.p;
-  }
+  ecc::Geometry g{};
+  g.n_views = n_views;
+  g.W = W;
+  g.H = H;
+  g.P = P;
+  g.motion = motion;
+  g.views = (ecc::ViewRec*)c->views.p;
+  g.status = c->d_status;
+  g.tan = grad ? (ecc::ViewTan*)c->vtan.p : nullptr;
+  g.tanP = grad_P ? (ecc::ViewTanP*)c->vtanP.p : nullptr;
+  g.n_alpha = n_alpha;
+  const bool new_grid = c->adir_n != n_alpha || c->adir_ptr != c->adir.p;  // the table depends on n_alpha only
+  g.alpha_dir = new_grid ? (float4*)c->adir.p : nullptr;
+  if ((e = ecc::launch_geometry(g, hk, s)) != cudaSuccess) return cuda_fail(c, e, "geometry launch");
+  c->adir_n = n_alpha;
+  c->adir_ptr = c->adir.p;
   // One pair set-up launch, then one pair-kernel launch, on the caller's stream.  (Set-up
   // chunks on a second stream beside the pair kernel's chunks were measured slower: the
   // two kernels sharing SMs slowed each other, 0.707 -> 0.765 ms on the 496-view scan.)
@@ -290,11 +301,6 @@ int run_evaluate(ecc_ctx* c, int n_views, const double* P, const double* motion,
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "pair q gradient launch");
   }
   if (grad) {
-    hk.on_begin("view_tangent_kernel", s);
-    ecc::view_tangent_kernel<<<(6 * n_views + 95) / 96, 96, 0, s>>>(n_views, P, motion, W, H,
-                                                                   (ecc::ViewTan*)c->vtan.p);
-    hk.on_end("view_tangent_kernel", s);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "view tangent launch");
     hk.on_begin("view_grad_theta_kernel", s);
     ecc::view_grad_theta_kernel<<<n_views, 256, 0, s>>>(n_views, np, pairs, (const float2*)c->gq.p,
                                                         (const ecc::ViewTan*)c->vtan.p, grad);
@@ -302,11 +308,6 @@ int run_evaluate(ecc_ctx* c, int n_views, const double* P, const double* motion,
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "gradient reduce launch");
   }
   if (grad_P) {
-    hk.on_begin("view_tangent_P_kernel", s);
-    ecc::view_tangent_P_kernel<<<(12 * n_views + 95) / 96, 96, 0, s>>>(n_views, P, motion, W, H,
-                                                                       (ecc::ViewTanP*)c->vtanP.p);
-    hk.on_end("view_tangent_P_kernel", s);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "view P tangent launch");
     hk.on_begin("view_grad_P_kernel", s);
     ecc::view_grad_P_kernel<<<n_views, 256, 0, s>>>(n_views, np, pairs, (const float2*)c->gq.p,
                                                     (const ecc::ViewTanP*)c->vtanP.p, grad_P);

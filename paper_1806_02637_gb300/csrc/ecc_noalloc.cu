@@ -122,12 +122,18 @@ extern "C" int ecc_evaluate_noalloc(int n_views, const double* P, const double* 
     e = cudaMemsetAsync(total, 0, sizeof(double), s);
     return e == cudaSuccess ? ECC_OK : fail(ECC_ECUDA, cudaGetErrorString(e));
   }
-  // the status word is OR-accumulated by the kernels: start it at zero
-  e = cudaMemsetAsync(status, 0, sizeof(int), s);
-  if (e != cudaSuccess) return fail(ECC_ECUDA, cudaGetErrorString(e));
   const ecc::LaunchHooks hk;  // no context: nothing to count or time
-  ecc::view_setup_kernel<<<(n_views + 127) / 128, 128, 0, s>>>(n_views, P, motion, W, H, views, status);
-  ecc::alpha_dir_kernel<<<(n_alpha + 255) / 256, 256, 0, s>>>(n_alpha, adir);
+  ecc::Geometry g{};
+  g.n_views = n_views;
+  g.W = W;
+  g.H = H;
+  g.P = P;
+  g.motion = motion;
+  g.views = views;
+  g.status = status;  // the kernels set bits there; this entry point reports none
+  g.n_alpha = n_alpha;
+  g.alpha_dir = adir;
+  if ((e = ecc::launch_geometry(g, hk, s)) != cudaSuccess) return fail(ECC_ECUDA, cudaGetErrorString(e));
   ecc::pair_setup_kernel<<<(n_pairs + 127) / 128, 128, 0, s>>>(n_views, 0, n_pairs, pairs, views, W, H, n_kappa, prs,
                                                                ctile, n_tiles, 0, status);
   if ((e = cudaGetLastError()) != cudaSuccess) return fail(ECC_ECUDA, cudaGetErrorString(e));

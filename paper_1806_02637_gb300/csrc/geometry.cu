@@ -1,9 +1,10 @@
 // Per-view and per-pair set-up of the ECC path (no matrix inverse anywhere): FP64 per
 // view, double-float (about 48 bits, on the FP32 pipes) per pair.
 //
-//  view_setup_kernel  one thread per view: rigid motion P' = P T(theta), scaling,
+//  geometry_kernel    one thread per view: rigid motion P' = P T(theta), scaling,
 //                     source as the meet of the rows of P (Eq. 4/5), cofactor
-//                     matrix, intrinsics.
+//                     matrix, intrinsics; in the same launch the views' tangents for
+//                     the gradients, the alpha-row directions and the line table.
 //  pair_setup_kernel  one thread per pair: pencil frame around the baseline, the
 //                     3x2 maps kappa -> epipolar line (the inverse-free form of
 //                     Eq. 13/14), valid arcs from the detector corners, the sampled
@@ -19,198 +20,311 @@ namespace ecc {
 
 namespace {
 
-template <class T>
-__host__ __device__ inline void cross3(const T* a, const T* b, T* c) {
-  c[0] = a[1] * b[2] - a[2] * b[1];
-  c[1] = a[2] * b[0] - a[0] * b[2];
-  c[2] = a[0] * b[1] - a[1] * b[0];
-}
-template <class T>
-__host__ __device__ inline T dot3(const T* a, const T* b) {
-  return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
-}
 __host__ __device__ inline void sc_pair(double x, double* s, double* c) { sincos(x, s, c); }
 template <int N>
 __device__ inline void sc_pair(const Dual<N>& x, Dual<N>* s, Dual<N>* c) { sincos(x, s, c); }
 
-// P T(theta), T = [R t; 0 1], R = Rz(rz) Ry(ry) Rx(rx).
-template <class TP, class T>
-__host__ __device__ void moved_projection(const TP* P, const T* th, T* out) {
-  T sx, cx, sy, cy, sz, cz;
-  sc_pair(th[0], &sx, &cx);
-  sc_pair(th[1], &sy, &cy);
-  sc_pair(th[2], &sz, &cz);
-  const T R[9] = {cz * cy, cz * sy * sx - sz * cx, cz * sy * cx + sz * sx,
-                  sz * cy, sz * sy * sx + cz * cx, sz * sy * cx - cz * sx,
-                  -sy,     cy * sx,                cy * cx};
-  for (int i = 0; i < 3; ++i) {
-    const TP* p = P + 4 * i;
-    for (int j = 0; j < 3; ++j) out[4 * i + j] = p[0] * R[j] + p[1] * R[3 + j] + p[2] * R[6 + j];
-    out[4 * i + 3] = p[0] * th[3] + p[1] * th[4] + p[2] * th[5] + T(p[3]);
+// A view's geometry while its lanes work on it.
+template <class T>
+struct ViewWork {
+  T sc[6];   // sin, cos of the motion's angles
+  T R[9];
+  T Pm[12];  // P T(theta)
+  T V[30];   // scaled P; 15 minors of its rows; (W - 1) / 2, (H - 1) / 2, 1
+  T S[11];   // X0 .. X3, u0, v0, m1.m1, |m3 x m1|^2, centred third cofactor row
+  T q[15];   // C, up, cofc
+  T D;
+  __host__ __device__ const T& u0() const { return S[4]; }
+  __host__ __device__ const T& v0() const { return S[5]; }
+};
+
+// Minor k of the rows of P, x[i] y[j] - x[j] y[i]: p, q, r, s, t, u of rows 1 and 2 (Eq. 5's
+// Pluecker coordinates), then the cofactor rows m2 x m3, m3 x m1, m1 x m2.
+__host__ __device__ inline int minor_code(int k) {  // x, y, i, j in two bits each
+#define ECC_M(x, y, i, j) ((unsigned long long)((x) | (y) << 2 | (i) << 4 | (j) << 6))
+  constexpr unsigned long long lo = ECC_M(0, 1, 2, 3) | ECC_M(0, 1, 1, 3) << 8 | ECC_M(0, 1, 1, 2) << 16 |
+                                    ECC_M(0, 1, 0, 3) << 24 | ECC_M(0, 1, 0, 2) << 32 | ECC_M(0, 1, 0, 1) << 40 |
+                                    ECC_M(1, 2, 1, 2) << 48 | ECC_M(1, 2, 2, 0) << 56;
+  constexpr unsigned long long hi = ECC_M(1, 2, 0, 1) | ECC_M(2, 0, 1, 2) << 8 | ECC_M(2, 0, 2, 0) << 16 |
+                                    ECC_M(2, 0, 0, 1) << 24 | ECC_M(0, 1, 1, 2) << 32 | ECC_M(0, 1, 2, 0) << 40 |
+                                    ECC_M(0, 1, 0, 1) << 48;
+#undef ECC_M
+  return (int)((k < 8 ? lo >> (8 * k) : hi >> (8 * (k - 8))) & 255);
+}
+
+// Sum k of three products of V: the source's homogeneous coordinates, the dot products, the
+// centred third cofactor row.  One product: sign, two places in V.
+__host__ __device__ inline unsigned long long sum_code(int k) {
+#define ECC_P(neg, i, j) ((unsigned long long)((neg) << 10 | (i) << 5 | (j)))
+#define ECC_S(p0, p1, p2) ((p0) | (p1) << 11 | (p2) << 22)
+  switch (k) {
+    case 0: return ECC_S(ECC_P(0, 12, 9), ECC_P(1, 13, 10), ECC_P(0, 14, 11));
+    case 1: return ECC_S(ECC_P(1, 12, 8), ECC_P(0, 15, 10), ECC_P(1, 16, 11));
+    case 2: return ECC_S(ECC_P(0, 13, 8), ECC_P(1, 15, 9), ECC_P(0, 17, 11));
+    case 3: return ECC_S(ECC_P(1, 14, 8), ECC_P(0, 16, 9), ECC_P(1, 17, 10));
+    case 4: return ECC_S(ECC_P(0, 0, 8), ECC_P(0, 1, 9), ECC_P(0, 2, 10));
+    case 5: return ECC_S(ECC_P(0, 4, 8), ECC_P(0, 5, 9), ECC_P(0, 6, 10));
+    case 6: return ECC_S(ECC_P(0, 0, 0), ECC_P(0, 1, 1), ECC_P(0, 2, 2));
+    case 7: return ECC_S(ECC_P(0, 21, 21), ECC_P(0, 22, 22), ECC_P(0, 23, 23));
+    default: {
+      const int c = k - 8;
+      return ECC_S(ECC_P(0, 27, 18 + c), ECC_P(0, 28, 21 + c), ECC_P(0, 29, 24 + c));
+    }
+  }
+#undef ECC_S
+#undef ECC_P
+}
+
+// Per-view geometry, by L lanes: the moved matrix P T(theta), T = [R t; 0 1],
+// R = Rz(rz) Ry(ry) Rx(rx); scaled P (third row of M unit, det M > 0), source as the meet of
+// the rows (Eq. 4, then Eq. 5 with p entering with the opposite sign), up axis m3 x m1,
+// cofactor rows (m2 x m3, m3 x m1, m1 x m2; l = cof(M) n) with the third row for centred
+// detector coordinates, principal point and source-detector distance.  Returns false (in
+// every lane) for a degenerate P.
+//
+// P(k) and th(k) give the matrix and the motion; sync() makes the lanes' stores to w visible
+// to each other.  T is double, or Dual for tangents.  One lane alone (L = 1, the host)
+// computes the same.  By lanes because an FP64 instruction holds its pipe 16 cycles and a
+// dependent one waits far longer: one thread's 1570 instructions per view took 10 us however
+// few the views (two views: launch of 15.3 us by threads, 11.6 us by lanes; 248 views and
+// their motion tangents: 20.7 + 22.5 us in two launches, 18.0 us in this one).
+template <int L, class T, class FP, class FT, class Sync>
+__host__ __device__ bool view_geometry(FP P, FT th, bool moved, int W, int H, int lane, ViewWork<T>& w, Sync sync) {
+  if (moved) {
+    for (int k = lane; k < 3; k += L) sc_pair(th(k), &w.sc[2 * k], &w.sc[2 * k + 1]);
+    sync();
+    for (int k = lane; k < 9; k += L) {
+      const int r = k / 3, c = k % 3;
+      const T sx = w.sc[0], cx = w.sc[1], sy = w.sc[2], cy = w.sc[3], sz = w.sc[4], cz = w.sc[5];
+      const T x = r == 0 ? cz : sz;
+      const T a = r == 2 ? cy : x * sy, e = r == 0 ? -sz : (r == 1 ? cz : T(0.0));
+      w.R[k] = c == 0 ? (r == 2 ? -sy : x * cy) : (c == 1 ? a * sx + e * cx : a * cx - e * sx);
+    }
+    sync();
+  }
+  for (int k = lane; k < 12; k += L) {
+    if (moved) {
+      const int i = k & ~3, j = k & 3;
+      const T x = j < 3 ? w.R[j] : th(3), y = j < 3 ? w.R[3 + j] : th(4), z = j < 3 ? w.R[6 + j] : th(5);
+      const T s = P(i) * x + P(i + 1) * y + P(i + 2) * z;
+      w.Pm[k] = j < 3 ? s : s + T(P(k));
+    } else {
+      w.Pm[k] = T(P(k));
+    }
+  }
+  if (lane == 0) {
+    w.V[27] = T(0.5 * (W - 1));
+    w.V[28] = T(0.5 * (H - 1));
+    w.V[29] = T(1.0);
+  }
+  sync();
+  const T* m1 = w.Pm;
+  const T* m2 = w.Pm + 4;
+  const T* m3 = w.Pm + 8;
+  const T det = m1[0] * (m2[1] * m3[2] - m2[2] * m3[1]) + m1[1] * (m2[2] * m3[0] - m2[0] * m3[2]) +
+                m1[2] * (m2[0] * m3[1] - m2[1] * m3[0]);
+  const T n3 = sqrt(m3[0] * m3[0] + m3[1] * m3[1] + m3[2] * m3[2]);
+  bool ok = isfinite(value(det)) && isfinite(value(n3)) && value(det) != 0.0 && value(n3) > 0.0;
+  for (int k = 0; k < 12; ++k) ok = ok && isfinite(value(w.Pm[k]));  // NaN / Inf anywhere, the motion's included
+  const T sc = ok ? T(copysign(1.0, value(det))) / n3 : T(0.0);
+  for (int k = lane; k < 12; k += L) w.V[k] = w.Pm[k] * sc;
+  sync();
+  for (int k = lane; k < 15; k += L) {
+    const int m = minor_code(k);
+    const T* x = w.V + 4 * (m & 3);
+    const T* y = w.V + 4 * (m >> 2 & 3);
+    const int i = m >> 4 & 3, j = m >> 6;
+    w.V[12 + k] = x[i] * y[j] - x[j] * y[i];
+  }
+  sync();
+  for (int k = lane; k < 11; k += L) {
+    const unsigned long long m = sum_code(k);
+    T x[3];
+    for (int i = 0; i < 3; ++i) {
+      x[i] = w.V[m >> (11 * i + 5) & 31];
+      if (m >> (11 * i + 10) & 1) x[i] = -x[i];
+    }
+    w.S[k] = x[0] * w.V[m & 31] + x[1] * w.V[m >> 11 & 31] + x[2] * w.V[m >> 22 & 31];
+  }
+  sync();
+  ok = ok && value(w.S[3]) != 0.0;
+  const T iw = ok ? T(1.0) / w.S[3] : T(0.0);
+  const T nu = sqrt(w.S[7]);
+  ok = ok && value(nu) > 0.0;
+  for (int k = lane; k < 15; k += L)
+    w.q[k] = k < 3 ? w.S[k] * iw : (k < 6 ? (ok ? w.V[18 + k] / nu : T(0.0)) : (k < 12 ? w.V[12 + k] : w.S[k - 4]));
+  const T dd = w.S[6] - w.S[4] * w.S[4];
+  ok = ok && value(dd) > 0.0;
+  const T D = ok ? sqrt(dd) : T(0.0);
+  if (lane == 0) w.D = D;
+  sync();
+  for (int k = 0; k < 3; ++k) ok = ok && isfinite(value(w.q[k]));
+  return ok;
+}
+
+// The view's record from its finished geometry, written by its lanes.
+template <int L>
+__host__ __device__ void write_view(const ViewWork<double>& w, bool ok, int lane, ViewRec* out) {
+  for (int k = lane; k < 15; k += L) {
+    if (k < 12) out->P[k] = w.V[k];
+    (k < 3 ? out->C[k] : (k < 6 ? out->up[k - 3] : out->cofc[k - 6])) = w.q[k];
+    const df q = df_from_double(w.q[k]);
+    out->qdf[2 * k] = q.hi;
+    out->qdf[2 * k + 1] = q.lo;
+  }
+  if (lane == 0) {
+    out->u0 = w.u0();
+    out->v0 = w.v0();
+    out->D = w.D;
+    out->status = ok ? 0 : 1;
+    out->pad = 0;
   }
 }
 
-// Per-view geometry from a (moved) projection matrix: scaled P (third row of M
-// unit, det M > 0), source as the meet of the rows (Eq. 4, then Eq. 5 with p
-// entering with the opposite sign), up axis m3 x m1, cofactor rows (m2 x m3,
-// m3 x m1, m1 x m2; l = cof(M) n) with the third row for centred detector
-// coordinates, principal point and source-detector distance.  Returns false for
-// a degenerate P.
-template <class T>
-__host__ __device__ bool view_geometry(const T* Pm, int W, int H, T* Pn, T* C, T* up, T* cofc, T* u0, T* v0, T* D) {
-  T m1[3] = {Pm[0], Pm[1], Pm[2]}, m2[3] = {Pm[4], Pm[5], Pm[6]}, m3[3] = {Pm[8], Pm[9], Pm[10]};
-  T c23[3];
-  cross3(m2, m3, c23);
-  const T det = dot3(m1, c23);
-  const T n3 = sqrt(dot3(m3, m3));
-  bool ok = isfinite(value(det)) && isfinite(value(n3)) && value(det) != 0.0 && value(n3) > 0.0;
-  for (int k = 0; k < 12; ++k) ok = ok && isfinite(value(Pm[k]));  // NaN / Inf anywhere, the motion's included
-  const T sc = ok ? T(copysign(1.0, value(det))) / n3 : T(0.0);
-  for (int k = 0; k < 12; ++k) Pn[k] = Pm[k] * sc;
-  const T* a = Pn;
-  const T* b = Pn + 4;
-  const T* c = Pn + 8;
-  const T p_ = a[2] * b[3] - a[3] * b[2], q_ = a[1] * b[3] - a[3] * b[1], r_ = a[1] * b[2] - a[2] * b[1];
-  const T s_ = a[0] * b[3] - a[3] * b[0], t_ = a[0] * b[2] - a[2] * b[0], u_ = a[0] * b[1] - a[1] * b[0];
-  const T X0 = p_ * c[1] - q_ * c[2] + r_ * c[3];
-  const T X1 = -p_ * c[0] + s_ * c[2] - t_ * c[3];
-  const T X2 = q_ * c[0] - s_ * c[1] + u_ * c[3];
-  const T X3 = -r_ * c[0] + t_ * c[1] - u_ * c[2];
-  ok = ok && value(X3) != 0.0;
-  const T iw = ok ? T(1.0) / X3 : T(0.0);
-  C[0] = X0 * iw;
-  C[1] = X1 * iw;
-  C[2] = X2 * iw;
-  T n1[3] = {Pn[0], Pn[1], Pn[2]}, n2[3] = {Pn[4], Pn[5], Pn[6]}, nn3[3] = {Pn[8], Pn[9], Pn[10]};
-  T upr[3];
-  cross3(nn3, n1, upr);
-  const T nu = sqrt(dot3(upr, upr));
-  ok = ok && value(nu) > 0.0;
-  for (int k = 0; k < 3; ++k) up[k] = ok ? upr[k] / nu : T(0.0);
-  T k0[3], k1[3], k2[3];
-  cross3(n2, nn3, k0);
-  cross3(nn3, n1, k1);
-  cross3(n1, n2, k2);
-  const double cxd = 0.5 * (W - 1), cyd = 0.5 * (H - 1);
-  for (int k = 0; k < 3; ++k) {
-    cofc[k] = k0[k];
-    cofc[3 + k] = k1[k];
-    cofc[6 + k] = cxd * k0[k] + cyd * k1[k] + k2[k];
+// Lanes per view, and per tangent direction: the FP64 pipe's time per direction falls with
+// fewer lanes, the chain of dependent instructions grows.
+constexpr int kViewLanes = 16, kTanLanes = 8;
+
+union GeometryShared {
+  ViewWork<double> view[32 / kViewLanes];
+  ViewWork<Dual<1>> tan[32 / kTanLanes];
+  __device__ GeometryShared() {}
+};
+
+// View i (of n) by its kViewLanes of the warp; lanes past the end work on the last view and
+// write nothing.  P and motion (or NULL) are the view's own.
+__device__ const ViewWork<double>& device_view(const double* __restrict__ P, const double* __restrict__ motion, int W,
+                                               int H, GeometryShared& sh, bool write, ViewRec* out, int* status) {
+  const int lane = threadIdx.x % kViewLanes;
+  ViewWork<double>& w = sh.view[threadIdx.x / kViewLanes];
+  const bool ok = view_geometry<kViewLanes, double>([=](int k) { return P[k]; }, [=](int k) { return motion[k]; },
+                                                    motion != nullptr, W, H, lane, w, [] { __syncwarp(); });
+  if (write) {
+    write_view<kViewLanes>(w, ok, lane, out);
+    if (!ok && lane == 0) atomicOr(status, kStatusDegenerateView);
   }
-  *u0 = dot3(n1, nn3);
-  *v0 = dot3(n2, nn3);
-  const T dd = dot3(n1, n1) - *u0 * *u0;
-  ok = ok && value(dd) > 0.0;
-  *D = ok ? sqrt(dd) : T(0.0);
-  for (int k = 0; k < 3; ++k) ok = ok && isfinite(value(C[k]));
-  return ok;
+  return w;
+}
+
+// Tangents of the per-view geometry q = (C, up, cofc), forward mode in FP64, one direction
+// per kTanLanes of the warp: with respect to motion parameter j (out[15][6], ViewTan) or,
+// WRT_P, to entry j of the unmoved P (out[15][12], ViewTanP; the view uses P T(theta)).  A
+// degenerate view's pairs carry no gradient; zero tangents keep its row at 0 (its NaN / Inf
+// geometry would otherwise turn 0 x tangent into NaN).
+template <bool WRT_P>
+__device__ void device_tangent(const double* __restrict__ P, const double* __restrict__ motion, int j, int W, int H,
+                               GeometryShared& sh, bool write, double* __restrict__ out) {
+  using D1 = Dual<1>;
+  const int lane = threadIdx.x % kTanLanes;
+  ViewWork<D1>& w = sh.tan[threadIdx.x / kTanLanes];
+  auto seeded = [](double x, bool one) {
+    D1 d(x);
+    d.d[0] = one ? 1.0 : 0.0;
+    return d;
+  };
+  auto th = [=](int k) { return seeded(motion ? motion[k] : 0.0, !WRT_P && k == j); };
+  bool ok;
+  if (WRT_P)
+    ok = view_geometry<kTanLanes, D1>([=](int k) { return seeded(P[k], k == j); }, th, motion != nullptr, W, H, lane, w,
+                                      [] { __syncwarp(); });
+  else
+    ok = view_geometry<kTanLanes, D1>([=](int k) { return P[k]; }, th, true, W, H, lane, w, [] { __syncwarp(); });
+  if (write)
+    for (int k = lane; k < 15; k += kTanLanes) out[(WRT_P ? 12 : 6) * k + j] = ok ? w.q[k].d[0] : 0.0;
+}
+
+// Line parameters of alpha row m of the Joseph line sums, as 32.32 fixed-point coordinates
+// along the interpolation axis (the x axis for rows, the y axis for columns).
+__device__ RadonRow radon_row(int m, int W, int H, int n_alpha, int n_s) {
+  constexpr double kTwo32 = 4294967296.0;
+  double sa, ca;
+  sincospi((double)m / (double)n_alpha, &sa, &ca);
+  const bool rows = (4 * m <= n_alpha) || (4 * m >= 3 * n_alpha);
+  const double ds = sqrt((double)W * W + (double)H * H) / (n_s - 1);
+  const double cx = 0.5 * (W - 1), cy = 0.5 * (H - 1);
+  const double p = rows ? ca : sa, q = rows ? sa : ca, cp = rows ? cx : cy, cq = rows ? cy : cx;
+  RadonRow r;
+  r.B0 = llrint((cp + (cq * q - 0.5 * n_s * ds) / p) * kTwo32);
+  r.STEP = llrint(ds / p * kTwo32);
+  r.DY = llrint(-q / p * kTwo32);
+  r.inv_len = (float)(1.0 / fabs(p));
+  r.ca = (float)ca;
+  r.sa = (float)sa;
+  r.rows_mode = rows ? 1 : 0;
+  return r;
 }
 
 }  // namespace
 
-__host__ __device__ ViewRec setup_view(const double* P, const double* motion, int W, int H) {
-  double Pm[12];
-  if (motion) {
-    moved_projection(P, motion, Pm);
-  } else {
-    for (int k = 0; k < 12; ++k) Pm[k] = P[k];
-  }
-  ViewRec r;
-  r.pad = 0;
-  const bool ok = view_geometry(Pm, W, H, r.P, r.C, r.up, r.cofc, &r.u0, &r.v0, &r.D);
-  r.status = ok ? 0 : 1;
-  for (int k = 0; k < 15; ++k) {
-    const df q = df_from_double(k < 3 ? r.C[k] : (k < 6 ? r.up[k - 3] : r.cofc[k - 6]));
-    r.qdf[2 * k] = q.hi;
-    r.qdf[2 * k + 1] = q.lo;
-  }
-  return r;
-}
+// All FP64 work of a call that depends on its geometry alone, in one launch: blocks of one
+// warp take views, tangent directions, alpha rows or table rows, by ranges of the block
+// index.  One warp per block because the FP64 pipe of an SM is what they would share.  (Set-up
+// and line table of two views: 14.4 + 13.9 us in two launches, 10.4 us in this one.)
+struct GeometryRanges {
+  int views, tan, tanP, alpha, table;  // blocks of each kind
+};
 
-__global__ void view_setup_kernel(int n_views, const double* __restrict__ P, const double* __restrict__ motion,
-                                  int W, int H, ViewRec* __restrict__ out, int* __restrict__ status) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_views) return;
-  const ViewRec r = setup_view(P + 12 * i, motion ? motion + 6 * i : nullptr, W, H);
-  if (r.status) atomicOr(status, kStatusDegenerateView);
-  out[i] = r;
-}
-
-// Tangents of the per-view geometry with respect to the view's own motion
-// parameters (forward mode, FP64): d C / d theta, d up / d theta, d cofc / d theta.
-__device__ ViewTan view_tangent(const double* P, const double* motion, int W, int H) {
-  using D6 = Dual<6>;
-  D6 th[6];
-  for (int j = 0; j < 6; ++j) {
-    th[j] = D6(motion ? motion[j] : 0.0);
-    th[j].d[j] = 1.0;
-  }
-  D6 Pm[12], Pn[12], C[3], up[3], cofc[9], u0, v0, D;
-  moved_projection(P, th, Pm);
-  // a degenerate view's pairs carry no gradient; zero tangents keep its row at 0
-  // (its NaN / Inf geometry would otherwise turn 0 x tangent into NaN)
-  const double ok = view_geometry(Pm, W, H, Pn, C, up, cofc, &u0, &v0, &D) ? 1.0 : 0.0;
-  ViewTan t;
-  for (int j = 0; j < 6; ++j) {
-    for (int k = 0; k < 3; ++k) {
-      t.dC[k][j] = ok ? C[k].d[j] : 0.0;
-      t.dup[k][j] = ok ? up[k].d[j] : 0.0;
+__global__ void __launch_bounds__(32) geometry_kernel(Geometry g, GeometryRanges n) {
+  __shared__ GeometryShared sh;
+  int b = (int)blockIdx.x;
+  if (b < n.views) {
+    const int i = b * (32 / kViewLanes) + threadIdx.x / kViewLanes;
+    const int v = min(i, g.n_views - 1);
+    const bool write = i < g.n_views;
+    const ViewWork<double>& w = device_view(g.P + 12 * v, g.motion ? g.motion + 6 * v : nullptr, g.W, g.H, sh, write,
+                                            g.views + v, g.status);
+    if (g.weights && write && threadIdx.x % kViewLanes == 0) {
+      RadonView o;
+      o.u0 = (float)w.u0();
+      o.v0 = (float)w.v0();
+      o.D = (float)w.D;
+      o.pad = 0;
+      g.weights[v] = o;
     }
-    for (int k = 0; k < 9; ++k) t.dcofc[k][j] = ok ? cofc[k].d[j] : 0.0;
+    return;
   }
-  return t;
+  b -= n.views;
+  if (b < n.tan) {
+    const long long i = (long long)b * (32 / kTanLanes) + threadIdx.x / kTanLanes, last = 6ll * g.n_views - 1;
+    const int v = (int)(min(i, last) / 6), j = (int)(min(i, last) % 6);
+    device_tangent<false>(g.P + 12 * v, g.motion ? g.motion + 6 * v : nullptr, j, g.W, g.H, sh, i <= last,
+                          &g.tan[v].dC[0][0]);
+    return;
+  }
+  b -= n.tan;
+  if (b < n.tanP) {
+    const long long i = (long long)b * (32 / kTanLanes) + threadIdx.x / kTanLanes, last = 12ll * g.n_views - 1;
+    const int v = (int)(min(i, last) / 12), j = (int)(min(i, last) % 12);
+    device_tangent<true>(g.P + 12 * v, g.motion ? g.motion + 6 * v : nullptr, j, g.W, g.H, sh, i <= last,
+                         &g.tanP[v].d[0][0]);
+    return;
+  }
+  b -= n.tanP;
+  if (b < n.alpha) {
+    const int m = 32 * b + threadIdx.x;
+    if (m >= g.n_alpha) return;
+    double s, c;
+    sincospi((double)m / (double)g.n_alpha, &s, &c);
+    g.alpha_dir[m] = split_dir(c, s);
+    return;
+  }
+  b -= n.alpha;
+  const long long i = 32ll * b + threadIdx.x;
+  if (i < (long long)g.copies * g.n_alpha) g.table[i] = radon_row((int)(i % g.n_alpha), g.W, g.H, g.n_alpha, g.n_s);
 }
 
-// The same tangents, one thread per (view, motion parameter j): column j of the
-// view's ViewTan (a single tangent direction, six times the threads of one Dual<6>
-// per view).
-__global__ void view_tangent_kernel(int n_views, const double* __restrict__ P, const double* __restrict__ motion,
-                                    int W, int H, ViewTan* __restrict__ out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 6LL * n_views) return;
-  const int lam = (int)(i / 6), j = (int)(i % 6);
-  using D1 = Dual<1>;
-  D1 th[6];
-  for (int k = 0; k < 6; ++k) th[k] = D1(motion ? motion[6 * lam + k] : 0.0);
-  th[j].d[0] = 1.0;
-  D1 Pm[12], Pn[12], C[3], up[3], cofc[9], u0, v0, D;
-  moved_projection(P + 12 * lam, th, Pm);
-  // a degenerate view's pairs carry no gradient; zero tangents keep its row at 0
-  const bool ok = view_geometry(Pm, W, H, Pn, C, up, cofc, &u0, &v0, &D);
-  ViewTan& t = out[lam];
-  for (int k = 0; k < 3; ++k) {
-    t.dC[k][j] = ok ? C[k].d[0] : 0.0;
-    t.dup[k][j] = ok ? up[k].d[0] : 0.0;
-  }
-  for (int k = 0; k < 9; ++k) t.dcofc[k][j] = ok ? cofc[k].d[0] : 0.0;
-}
-
-// Tangents of q = (C, up, cofc) with respect to the 12 entries of the unmoved P
-// (forward mode, FP64; the view uses P T(theta)): one thread per (view, entry j),
-// one tangent direction each.
-__global__ void view_tangent_P_kernel(int n_views, const double* __restrict__ P, const double* __restrict__ motion,
-                                      int W, int H, ViewTanP* __restrict__ out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 12LL * n_views) return;
-  const int lam = (int)(i / 12), j = (int)(i % 12);
-  using D1 = Dual<1>;
-  D1 Pd[12], Pm[12], Pn[12], C[3], up[3], cofc[9], u0, v0, D;
-  for (int k = 0; k < 12; ++k) Pd[k] = D1(P[12 * lam + k]);
-  Pd[j].d[0] = 1.0;
-  if (motion) {
-    D1 th[6];
-    for (int k = 0; k < 6; ++k) th[k] = D1(motion[6 * lam + k]);
-    moved_projection(Pd, th, Pm);
-  } else {
-    for (int k = 0; k < 12; ++k) Pm[k] = Pd[k];
-  }
-  const bool ok = view_geometry(Pm, W, H, Pn, C, up, cofc, &u0, &v0, &D);  // degenerate: zero tangents
-  ViewTanP& t = out[lam];
-  for (int k = 0; k < 3; ++k) {
-    t.d[k][j] = ok ? C[k].d[0] : 0.0;
-    t.d[3 + k][j] = ok ? up[k].d[0] : 0.0;
-  }
-  for (int k = 0; k < 9; ++k) t.d[6 + k][j] = ok ? cofc[k].d[0] : 0.0;
+cudaError_t launch_geometry(const Geometry& g, const LaunchHooks& hooks, cudaStream_t stream) {
+  auto blocks = [](bool on, long long n, int per) { return on ? (int)((n + per - 1) / per) : 0; };
+  GeometryRanges n;
+  n.views = blocks(g.views != nullptr, g.n_views, 32 / kViewLanes);
+  n.tan = blocks(g.tan != nullptr, 6ll * g.n_views, 32 / kTanLanes);
+  n.tanP = blocks(g.tanP != nullptr, 12ll * g.n_views, 32 / kTanLanes);
+  n.alpha = blocks(g.alpha_dir != nullptr, g.n_alpha, 32);
+  n.table = blocks(g.table != nullptr, (long long)g.copies * g.n_alpha, 32);
+  hooks.on_begin("geometry_kernel", stream);
+  geometry_kernel<<<n.views + n.tan + n.tanP + n.alpha + n.table, 32, 0, stream>>>(g, n);
+  hooks.on_end("geometry_kernel", stream);
+  return cudaGetLastError();
 }
 
 namespace {
@@ -695,17 +809,27 @@ __global__ void __launch_bounds__(256) view_grad_P_kernel(int n_views, long long
 }
 
 // ---------------------------------------------------------------- serving rounds
-__global__ void serve_view_kernel(const ServeJob* __restrict__ jobs, const long long* __restrict__ voff, int n_jobs,
-                                  long long total) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  const int j = serve_job_of(voff, n_jobs, i);
+// Blocks of one warp as in geometry_kernel: first the views, then (of jobs that take a
+// gradient step) the tangent directions.
+__global__ void __launch_bounds__(32) serve_view_kernel(const ServeJob* __restrict__ jobs,
+                                                        const long long* __restrict__ voff, int n_jobs, long long total,
+                                                        int view_blocks) {
+  __shared__ GeometryShared sh;
+  if ((int)blockIdx.x < view_blocks) {
+    const long long t = (long long)blockIdx.x * (32 / kViewLanes) + threadIdx.x / kViewLanes, i = min(t, total - 1);
+    const int j = serve_job_of(voff, n_jobs, i);
+    const ServeJob& J = jobs[j];
+    const long long v = i - voff[j];
+    device_view(J.P + 12 * v, J.theta + 6 * v, J.W, J.H, sh, t < total, J.views + v, J.status);
+    return;
+  }
+  const long long t = (long long)((int)blockIdx.x - view_blocks) * (32 / kTanLanes) + threadIdx.x / kTanLanes;
+  const long long i = min(t, 6 * total - 1) / 6;
+  const int j = serve_job_of(voff, n_jobs, i), dir = (int)(min(t, 6 * total - 1) % 6);
   const ServeJob& J = jobs[j];
+  if (!__any_sync(0xffffffffu, J.do_grad)) return;
   const long long v = i - voff[j];
-  const ViewRec r = setup_view(J.P + 12 * v, J.theta + 6 * v, J.W, J.H);
-  if (r.status) atomicOr(J.status, kStatusDegenerateView);
-  J.views[v] = r;
-  if (J.do_grad) J.vtan[v] = view_tangent(J.P + 12 * v, J.theta + 6 * v, J.W, J.H);
+  device_tangent<false>(J.P + 12 * v, J.theta + 6 * v, dir, J.W, J.H, sh, J.do_grad && t < 6 * total, &J.vtan[v].dC[0][0]);
 }
 
 __global__ void serve_pair_setup_kernel(const ServeJob* __restrict__ jobs, const long long* __restrict__ poff,
@@ -812,7 +936,12 @@ cudaError_t launch_serve_motion(const ServeJob* jobs, const long long* voff, int
 
 cudaError_t launch_serve_setup(const ServeJob* jobs, const long long* voff, const long long* poff, int n_jobs,
                                long long n_views, long long n_pairs, cudaStream_t stream) {
-  if (n_views > 0) serve_view_kernel<<<(unsigned)((n_views + 63) / 64), 64, 0, stream>>>(jobs, voff, n_jobs, n_views);
+  if (n_views > 0) {
+    const long long view_blocks = (n_views + 32 / kViewLanes - 1) / (32 / kViewLanes);
+    const long long tan_blocks = (6 * n_views + 32 / kTanLanes - 1) / (32 / kTanLanes);
+    serve_view_kernel<<<(unsigned)(view_blocks + tan_blocks), 32, 0, stream>>>(jobs, voff, n_jobs, n_views,
+                                                                               (int)view_blocks);
+  }
   if (n_pairs > 0)
     serve_pair_setup_kernel<<<(unsigned)((n_pairs + 127) / 128), 128, 0, stream>>>(jobs, poff, n_jobs, n_pairs);
   return cudaGetLastError();
@@ -830,14 +959,6 @@ cudaError_t launch_serve_grad(const ServeJob* jobs, const long long* voff, const
   return cudaGetLastError();
 }
 
-__global__ void alpha_dir_kernel(int n_alpha, float4* __restrict__ dir) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= n_alpha) return;
-  double s, c;
-  sincospi((double)m / (double)n_alpha, &s, &c);
-  dir[m] = split_dir(c, s);
-}
-
 }  // namespace ecc
 
 // Internal host entry point (tests only, not part of the public ABI): runs the
@@ -851,8 +972,14 @@ extern "C" int ecc_internal_setup_pair_host(int n_views, const double* P, const 
                                             int a, int b, double* info_out, double* A_out) {
   if (n_views < 1 || a < 0 || b < 0 || a >= n_views || b >= n_views || K < 1) return -1;
   ecc::ViewRec views[2];
-  views[0] = ecc::setup_view(P + 12 * a, motion ? motion + 6 * a : nullptr, W, H);
-  views[1] = ecc::setup_view(P + 12 * b, motion ? motion + 6 * b : nullptr, W, H);
+  for (int s = 0; s < 2; ++s) {
+    const double* p = P + 12 * (s ? b : a);
+    const double* m = motion ? motion + 6 * (s ? b : a) : nullptr;
+    ecc::ViewWork<double> w;
+    const bool ok = ecc::view_geometry<1, double>([=](int k) { return p[k]; }, [=](int k) { return m[k]; },
+                                                  m != nullptr, W, H, 0, w, [] {});
+    ecc::write_view<1>(w, ok, 0, &views[s]);
+  }
   const int n_tiles = (K + 31) / 32;
   float4* ct = new float4[n_tiles];
   const ecc::PairRec r = ecc::setup_pair(0, 1, 2, views, W, H, K, ct, n_tiles, nullptr);

@@ -8,22 +8,16 @@
 
 namespace ecc {
 
-__global__ void view_setup_kernel(int n_views, const double* P, const double* motion, int W, int H, ViewRec* out,
-                                  int* status);
 // pairs [p_begin, p_end) of the row-major a < b enumeration (pairs == NULL) or of the list
 __global__ void pair_setup_kernel(int n_views, long long p_begin, long long p_end, const int32_t* pairs,
                                   const ViewRec* views, int W, int H, int K, PairRec* out, float4* ctile, int n_tiles,
                                   int reuse_sampling, int* status);
-__global__ void view_tangent_kernel(int n_views, const double* P, const double* motion, int W, int H, ViewTan* out);
 __global__ void view_grad_theta_kernel(int n_views, long long n_pairs, const int32_t* pairs, const float2* gq,
                                        const ViewTan* vtan, double* grad);
-__global__ void view_tangent_P_kernel(int n_views, const double* P, const double* motion, int W, int H,
-                                      ViewTanP* out);
 __global__ void pair_grad_q_kernel(long long n_pairs, const PairRec* prs, const ViewRec* views, const double* Gpp,
                                    float2* gq);
 __global__ void view_grad_P_kernel(int n_views, long long n_pairs, const int32_t* pairs, const float2* gq,
                                    const ViewTanP* vtan, double* grad_P);
-__global__ void alpha_dir_kernel(int n_alpha, float4* dir);
 
 // Line parameters of the Joseph line sums at one alpha row (32.32 fixed point).
 struct RadonRow {
@@ -38,6 +32,23 @@ struct RadonRow {
 struct RadonView {  // per-view weights (FP32 copies of the FP64 set-up)
   float u0, v0, D;
   int pad;
+};
+
+// The FP64 work of a call that depends on its geometry alone, in one launch: what is not
+// wanted is NULL.
+struct Geometry {
+  int n_views, W, H;
+  const double* P;       // [n_views][12]
+  const double* motion;  // [n_views][6] or NULL
+  ViewRec* views;        // per-view set-up
+  int* status;
+  RadonView* weights;    // of the dRadon/ds precompute
+  ViewTan* tan;          // tangents with respect to the motion
+  ViewTanP* tanP;        // and with respect to P
+  int n_alpha, n_s;
+  float4* alpha_dir;     // alpha-row directions
+  RadonRow* table;       // line table of the precompute, `copies` times
+  int copies;
 };
 
 // Callbacks around every kernel launch (launch counting and optional CUDA-event
@@ -99,7 +110,14 @@ struct RadonPlan {
   int batch;           // views per pass over the scratch
   size_t wimg_bytes;   // weighted images
   size_t stage_bytes;  // FP32 staging of FP16 storage
-  size_t table_bytes(int n_views, int n_alpha) const;  // line table and per-view weights
+  // the line table (copies of n_alpha rows) and the per-view weights after it
+  int copies(int n_views) const { return views ? 1 : n_views; }
+  size_t table_bytes(int n_views, int n_alpha) const {
+    return sizeof(RadonRow) * (size_t)copies(n_views) * n_alpha + sizeof(RadonView) * (size_t)n_views;
+  }
+  RadonView* weights(RadonRow* table, int n_views, int n_alpha) const {
+    return reinterpret_cast<RadonView*>(table + (size_t)copies(n_views) * n_alpha);
+  }
 };
 // At most max_batch views per pass; wimg_cap bounds the many-view form's scratch and
 // total_cap (0: none) its scratch and staging together.  Where no group of views fits
@@ -116,8 +134,9 @@ struct ViewsPlan {
 };
 
 // Launchers (return cudaError_t of the launch).
-cudaError_t launch_radon(const ViewRec* views, int n_views, const float* images, int W, int H, int n_alpha, int n_s,
-                         int dtype, void* sino_out, float* scales_out, RadonRow* table, void* wimg, float* stage,
+cudaError_t launch_geometry(const Geometry& g, const LaunchHooks& hooks, cudaStream_t stream);
+cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_alpha, int n_s, int dtype,
+                         void* sino_out, float* scales_out, const RadonRow* table, void* wimg, float* stage,
                          const RadonPlan& plan, int* status, const LaunchHooks& hooks, cudaStream_t stream,
                          const cudaEvent_t* batch_ready = nullptr);  // per batch: wait before reading its images
 cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n_views, const float* images, int W,

@@ -1,10 +1,10 @@
 // dRadon/ds precompute: the Grangeat intermediate function S_lambda (Eq. 1) of
 // every projection on an (alpha, s) grid.
 //
-//   radon_table_kernel   FP64, one thread per alpha row (and view): the parameters of
-//                        the detector lines (x - cx) cos a + (y - cy) sin a = sigma
-//                        as 32.32 fixed-point coordinates along the interpolation
-//                        axis (exact integer stepping, no FP64 in the hot loop).
+//   line table           (FP64, geometry_kernel) the parameters of the detector lines
+//                        (x - cx) cos a + (y - cy) sin a = sigma as 32.32 fixed-point
+//                        coordinates along the interpolation axis (exact integer
+//                        stepping, no FP64 in the hot loop).
 //   weight_kernel        cosine pre-weight g D / sqrt(D^2 + u^2 + v^2) of each
 //                        projection, stored as interpolation pairs (v[i],
 //                        v[i+1] - v[i]) twice: along image rows and along image
@@ -30,55 +30,6 @@
 namespace ecc {
 
 namespace {
-
-constexpr double kTwo32 = 4294967296.0;
-
-// copies: the line parameters are the same for every view; the view-by-view form reads a
-// copy per view (its kernel, indexed so, compiles to 64 registers and four blocks per SM;
-// with one shared copy it takes 48, and the bands of five blocks thrash L1: 65 us against
-// 31 on two 256 x 256 views), the many-view form one.
-__global__ void radon_table_kernel(const ViewRec* __restrict__ views, int n_views, int copies, int W, int H,
-                                   int n_alpha, int n_s, RadonRow* __restrict__ table,
-                                   RadonView* __restrict__ rv) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < n_views) {
-    const ViewRec& vr = views[idx];
-    RadonView o;
-    o.u0 = (float)vr.u0;
-    o.v0 = (float)vr.v0;
-    o.D = (float)vr.D;
-    o.pad = 0;
-    rv[idx] = o;
-  }
-  if (idx >= (long long)copies * n_alpha) return;
-  const int m = (int)(idx % n_alpha);
-  double sa, ca;
-  sincospi((double)m / (double)n_alpha, &sa, &ca);
-  const bool rows = (4 * m <= n_alpha) || (4 * m >= 3 * n_alpha);
-  const double ds = sqrt((double)W * W + (double)H * H) / (n_s - 1);
-  const double cx = 0.5 * (W - 1), cy = 0.5 * (H - 1);
-  double B0, STEP, DY, inv_len;
-  if (rows) {
-    B0 = cx + (cy * sa - 0.5 * n_s * ds) / ca;
-    STEP = ds / ca;
-    DY = -sa / ca;
-    inv_len = 1.0 / fabs(ca);
-  } else {
-    B0 = cy + (cx * ca - 0.5 * n_s * ds) / sa;
-    STEP = ds / sa;
-    DY = -ca / sa;
-    inv_len = 1.0 / fabs(sa);
-  }
-  RadonRow r;
-  r.B0 = llrint(B0 * kTwo32);
-  r.STEP = llrint(STEP * kTwo32);
-  r.DY = llrint(DY * kTwo32);
-  r.inv_len = (float)inv_len;
-  r.ca = (float)ca;
-  r.sa = (float)sa;
-  r.rows_mode = rows ? 1 : 0;
-  table[idx] = r;
-}
 
 // Weighted projection as interpolation pairs (v[i], v[i+1] - v[i]) along the
 // interpolation axis: row-major [H][pitch_r] (pairs along x) and transposed
@@ -306,10 +257,6 @@ size_t radon_f16_stage_bytes(int n_alpha, int n_s, int batch_views) {
   return sizeof(float) * (size_t)n_alpha * n_s * batch_views;
 }
 
-size_t RadonPlan::table_bytes(int n_views, int n_alpha) const {
-  return sizeof(RadonRow) * (size_t)(views ? 1 : n_views) * n_alpha + sizeof(RadonView) * (size_t)n_views;
-}
-
 RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch, size_t wimg_cap,
                      size_t total_cap) {
   RadonPlan p{};
@@ -356,22 +303,11 @@ static cudaError_t quantize_batch(const float* stage, size_t per_view, int nb, f
   return cudaGetLastError();
 }
 
-cudaError_t launch_radon(const ViewRec* views, int n_views, const float* images, int W, int H, int n_alpha, int n_s,
-                         int dtype, void* sino_out, float* scales_out, RadonRow* table, void* wimg,
-                         float* stage, const RadonPlan& plan, int* status, const LaunchHooks& hooks,
-                         cudaStream_t stream, const cudaEvent_t* batch_ready) {
-  // table and per-view weights (RadonView array sits right after the table)
-  const int copies = plan.views ? 1 : n_views;
-  RadonView* rv = reinterpret_cast<RadonView*>(table + (size_t)copies * n_alpha);
-  {
-    const long long n = std::max((long long)n_views, (long long)copies * n_alpha);
-    hooks.on_begin("radon_table_kernel", stream);
-    radon_table_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(views, n_views, copies, W, H, n_alpha, n_s,
-                                                                       table, rv);
-    hooks.on_end("radon_table_kernel", stream);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_alpha, int n_s, int dtype,
+                         void* sino_out, float* scales_out, const RadonRow* table, void* wimg, float* stage,
+                         const RadonPlan& plan, int* status, const LaunchHooks& hooks, cudaStream_t stream,
+                         const cudaEvent_t* batch_ready) {
+  const RadonView* rv = plan.weights(const_cast<RadonRow*>(table), n_views, n_alpha);
   JosephArgs jg;
   jg.W = W;
   jg.H = H;

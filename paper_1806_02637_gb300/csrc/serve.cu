@@ -218,16 +218,27 @@ bool admit_job(ecc_serve* S, Job* J) {
     return false;
   }
   cudaEventRecord(S->admit_t[1], s);
-  ecc::view_setup_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(
-      (int)n, (const double*)(R + L.P), nullptr, d.W, d.H, (ecc::ViewRec*)(R + L.views), (int*)(R + L.status));
-  ecc::alpha_dir_kernel<<<(d.n_alpha + 255) / 256, 256, 0, s>>>(d.n_alpha, (float4*)(R + L.adir));
-  e = cudaGetLastError();
-  if (e == cudaSuccess) {
+  {
     const ecc::LaunchHooks hk;
-    e = ecc::launch_radon((const ecc::ViewRec*)(R + L.views), (int)n, (const float*)(T + L.images), d.W, d.H,
-                          d.n_alpha, d.n_s, d.dtype, R + L.sino, (float*)(R + L.scales),
-                          (ecc::RadonRow*)(T + L.rtable), T + L.wimg, (float*)(T + L.stage), L.plan,
-                          (int*)(R + L.status), hk, s);
+    ecc::RadonRow* table = (ecc::RadonRow*)(T + L.rtable);
+    ecc::Geometry g{};
+    g.n_views = (int)n;
+    g.W = d.W;
+    g.H = d.H;
+    g.P = (const double*)(R + L.P);
+    g.views = (ecc::ViewRec*)(R + L.views);
+    g.status = (int*)(R + L.status);
+    g.weights = L.plan.weights(table, (int)n, d.n_alpha);
+    g.n_alpha = d.n_alpha;
+    g.n_s = d.n_s;
+    g.alpha_dir = (float4*)(R + L.adir);
+    g.table = table;
+    g.copies = L.plan.copies((int)n);
+    e = ecc::launch_geometry(g, hk, s);
+    if (e == cudaSuccess)
+      e = ecc::launch_radon((int)n, (const float*)(T + L.images), d.W, d.H, d.n_alpha, d.n_s, d.dtype, R + L.sino,
+                            (float*)(R + L.scales), table, T + L.wimg, (float*)(T + L.stage), L.plan,
+                            (int*)(R + L.status), hk, s);
   }
   if (e != cudaSuccess) {
     set_err(J, ECC_ECUDA, cuda_msg("precompute launch", e));
