@@ -289,28 +289,30 @@ int run_evaluate(ecc_ctx* c, int n_views, const double* P, const double* motion,
                             per_pair, nkappa, (double*)c->partial.p, (grad || grad_P) ? (double*)c->Gpp.p : nullptr,
                             c->d_status, &nb, hk, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "pair kernel launch");
-  e = ecc::launch_reduce((const double*)c->partial.p, nb, total, hk, s);
-  if (e != cudaSuccess) return cuda_fail(c, e, "reduce launch");
-  if (grad || grad_P) {
-    // d e / d (C, up, cofc) per pair, shared by both gradients
+  if (!grad && !grad_P) {
+    e = ecc::launch_reduce((const double*)c->partial.p, nb, total, hk, s);
+    if (e != cudaSuccess) return cuda_fail(c, e, "reduce launch");
+  } else {
+    // d e / d (C, up, cofc) per pair, shared by both gradients, and the total
     hk.on_begin("pair_grad_q_kernel", s);
-    ecc::pair_grad_q_kernel<<<(unsigned)((np + 63) / 64), 64, 0, s>>>(np, (const ecc::PairRec*)c->pairs.p,
-                                                                      (const ecc::ViewRec*)c->views.p,
-                                                                      (const double*)c->Gpp.p, (float2*)c->gq.p);
+    const unsigned blocks = 1 + (unsigned)((np + ecc::kGradQThreads - 1) / ecc::kGradQThreads);
+    ecc::launch_behind(ecc::pair_grad_q_kernel, blocks, ecc::kGradQThreads, 0, s, np, (const ecc::PairRec*)c->pairs.p,
+                       (const ecc::ViewRec*)c->views.p, (const double*)c->Gpp.p, (float2*)c->gq.p,
+                       (const double*)c->partial.p, nb, total);
     hk.on_end("pair_grad_q_kernel", s);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "pair q gradient launch");
   }
   if (grad) {
     hk.on_begin("view_grad_theta_kernel", s);
-    ecc::view_grad_theta_kernel<<<n_views, 256, 0, s>>>(n_views, np, pairs, (const float2*)c->gq.p,
-                                                        (const ecc::ViewTan*)c->vtan.p, grad);
+    ecc::launch_behind(ecc::view_grad_theta_kernel, n_views, 256, 0, s, n_views, np, pairs, (const float2*)c->gq.p,
+                       (const ecc::ViewTan*)c->vtan.p, grad);
     hk.on_end("view_grad_theta_kernel", s);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "gradient reduce launch");
   }
   if (grad_P) {
     hk.on_begin("view_grad_P_kernel", s);
-    ecc::view_grad_P_kernel<<<n_views, 256, 0, s>>>(n_views, np, pairs, (const float2*)c->gq.p,
-                                                    (const ecc::ViewTanP*)c->vtanP.p, grad_P);
+    ecc::launch_behind(ecc::view_grad_P_kernel, n_views, 256, 0, s, n_views, np, pairs, (const float2*)c->gq.p,
+                       (const ecc::ViewTanP*)c->vtanP.p, grad_P);
     hk.on_end("view_grad_P_kernel", s);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "P gradient reduce launch");
   }

@@ -1137,26 +1137,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, GRAD ? 2 : 4) ecc_pair_ke
   pair_block<T, GRAD>(g, blockIdx.x, e_warp, recs, lps);
 }
 
-// Fixed-order sum of n block partials by one block of 1024 threads: deterministic.
-__device__ void reduce_fixed(const double* __restrict__ partial, int n, double* __restrict__ total, double* s) {
-  double acc = 0.0;
-  const int per = (n + blockDim.x - 1) / blockDim.x;
-  const int beg = threadIdx.x * per;
-  const int end = min(n, beg + per);
-  for (int i = beg; i < end; ++i) acc += partial[i];
-  s[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *total = s[0];
-}
-
+// The total of a call without gradients.
 __global__ void __launch_bounds__(1024) reduce_kernel(const double* __restrict__ partial, int n,
                                                       double* __restrict__ total) {
-  __shared__ double s[1024];
-  reduce_fixed(partial, n, total, s);
+  wait_for_previous();
+  __shared__ double s[kSumSlots];
+  reduce_fixed<1024>(partial, n, total, s);
 }
 
 // Serving: all active jobs' pair blocks in one persistent launch.  Each CTA takes
@@ -1196,9 +1182,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 3) serve_pair_kernel(cons
 }
 
 __global__ void __launch_bounds__(1024) serve_reduce_kernel(const ServeJob* __restrict__ jobs) {
-  __shared__ double s[1024];
+  __shared__ double s[kSumSlots];
   const ServeJob& J = jobs[blockIdx.x];
-  reduce_fixed(J.pair.block_partial, (int)((J.pair.n_pairs + kWarpsPerBlock - 1) / kWarpsPerBlock), J.total_out, s);
+  const int n_blocks = (int)((J.pair.n_pairs + kWarpsPerBlock - 1) / kWarpsPerBlock);
+  reduce_fixed<1024>(J.pair.block_partial, n_blocks, J.total_out, s);
 }
 
 }  // namespace
@@ -1281,7 +1268,7 @@ cudaError_t launch_serve_pairs(const ServeJob* jobs, const long long* boff, int 
 cudaError_t launch_reduce(const double* partial, int n, double* total, const LaunchHooks& hooks,
                           cudaStream_t stream) {
   hooks.on_begin("reduce_kernel", stream);
-  reduce_kernel<<<1, 1024, 0, stream>>>(partial, n, total);
+  launch_behind(reduce_kernel, 1, 1024, 0, stream, partial, n, total);
   hooks.on_end("reduce_kernel", stream);
   return cudaGetLastError();
 }

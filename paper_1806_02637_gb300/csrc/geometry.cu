@@ -24,6 +24,32 @@ __host__ __device__ inline void sc_pair(double x, double* s, double* c) { sincos
 template <int N>
 __device__ inline void sc_pair(const Dual<N>& x, Dual<N>* s, Dual<N>* c) { sincos(x, s, c); }
 
+// a b + c, one rounding on doubles: written out, so that the records do not depend on what the
+// compiler contracts.
+__host__ __device__ inline double mad(double a, double b, double c) { return fma(a, b, c); }
+template <int N>
+__host__ __device__ inline Dual<N> mad(const Dual<N>& a, const Dual<N>& b, const Dual<N>& c) {
+  return a * b + c;
+}
+template <int N>
+__host__ __device__ inline Dual<N> mad(double a, const Dual<N>& b, const Dual<N>& c) {
+  return a * b + c;
+}
+
+// a b - c d with one rounding less (fused), or all three.
+__host__ __device__ inline double cross2(double a, double b, double c, double d, bool fused) {
+#ifdef __CUDA_ARCH__
+  return fused ? fma(a, b, -__dmul_rn(c, d)) : __dsub_rn(__dmul_rn(a, b), __dmul_rn(c, d));
+#else
+  return fused ? fma(a, b, -(c * d)) : a * b - c * d;
+#endif
+}
+template <int N>
+__host__ __device__ inline Dual<N> cross2(const Dual<N>& a, const Dual<N>& b, const Dual<N>& c, const Dual<N>& d,
+                                          bool) {
+  return a * b - c * d;
+}
+
 // A view's geometry while its lanes work on it.
 template <class T>
 struct ViewWork {
@@ -38,12 +64,12 @@ struct ViewWork {
   __host__ __device__ const T& v0() const { return S[5]; }
 };
 
-// Minor k of the rows of P, x[i] y[j] - x[j] y[i]: p, q, r, s, t, u of rows 1 and 2 (Eq. 5's
+// Minor k of the rows of P, x[i] y[j] - x[j] y[i]: p, q, r, s, -t, u of rows 1 and 2 (Eq. 5's
 // Pluecker coordinates), then the cofactor rows m2 x m3, m3 x m1, m1 x m2.
 __host__ __device__ inline int minor_code(int k) {  // x, y, i, j in two bits each
 #define ECC_M(x, y, i, j) ((unsigned long long)((x) | (y) << 2 | (i) << 4 | (j) << 6))
   constexpr unsigned long long lo = ECC_M(0, 1, 2, 3) | ECC_M(0, 1, 1, 3) << 8 | ECC_M(0, 1, 1, 2) << 16 |
-                                    ECC_M(0, 1, 0, 3) << 24 | ECC_M(0, 1, 0, 2) << 32 | ECC_M(0, 1, 0, 1) << 40 |
+                                    ECC_M(0, 1, 0, 3) << 24 | ECC_M(0, 1, 2, 0) << 32 | ECC_M(0, 1, 0, 1) << 40 |
                                     ECC_M(1, 2, 1, 2) << 48 | ECC_M(1, 2, 2, 0) << 56;
   constexpr unsigned long long hi = ECC_M(1, 2, 0, 1) | ECC_M(2, 0, 1, 2) << 8 | ECC_M(2, 0, 2, 0) << 16 |
                                     ECC_M(2, 0, 0, 1) << 24 | ECC_M(0, 1, 1, 2) << 32 | ECC_M(0, 1, 2, 0) << 40 |
@@ -58,17 +84,17 @@ __host__ __device__ inline unsigned long long sum_code(int k) {
 #define ECC_P(neg, i, j) ((unsigned long long)((neg) << 10 | (i) << 5 | (j)))
 #define ECC_S(p0, p1, p2) ((p0) | (p1) << 11 | (p2) << 22)
   switch (k) {
-    case 0: return ECC_S(ECC_P(0, 12, 9), ECC_P(1, 13, 10), ECC_P(0, 14, 11));
-    case 1: return ECC_S(ECC_P(1, 12, 8), ECC_P(0, 15, 10), ECC_P(1, 16, 11));
-    case 2: return ECC_S(ECC_P(0, 13, 8), ECC_P(1, 15, 9), ECC_P(0, 17, 11));
-    case 3: return ECC_S(ECC_P(1, 14, 8), ECC_P(0, 16, 9), ECC_P(1, 17, 10));
-    case 4: return ECC_S(ECC_P(0, 0, 8), ECC_P(0, 1, 9), ECC_P(0, 2, 10));
-    case 5: return ECC_S(ECC_P(0, 4, 8), ECC_P(0, 5, 9), ECC_P(0, 6, 10));
-    case 6: return ECC_S(ECC_P(0, 0, 0), ECC_P(0, 1, 1), ECC_P(0, 2, 2));
-    case 7: return ECC_S(ECC_P(0, 21, 21), ECC_P(0, 22, 22), ECC_P(0, 23, 23));
+    case 0: return ECC_S(ECC_P(1, 13, 10), ECC_P(0, 12, 9), ECC_P(0, 14, 11));
+    case 1: return ECC_S(ECC_P(1, 12, 8), ECC_P(0, 15, 10), ECC_P(0, 16, 11));
+    case 2: return ECC_S(ECC_P(1, 15, 9), ECC_P(0, 13, 8), ECC_P(0, 17, 11));
+    case 3: return ECC_S(ECC_P(1, 14, 8), ECC_P(1, 16, 9), ECC_P(1, 17, 10));
+    case 4: return ECC_S(ECC_P(0, 1, 9), ECC_P(0, 0, 8), ECC_P(0, 2, 10));
+    case 5: return ECC_S(ECC_P(0, 5, 9), ECC_P(0, 4, 8), ECC_P(0, 6, 10));
+    case 6: return ECC_S(ECC_P(0, 1, 1), ECC_P(0, 0, 0), ECC_P(0, 2, 2));
+    case 7: return ECC_S(ECC_P(0, 22, 22), ECC_P(0, 21, 21), ECC_P(0, 23, 23));
     default: {
       const int c = k - 8;
-      return ECC_S(ECC_P(0, 27, 18 + c), ECC_P(0, 28, 21 + c), ECC_P(0, 29, 24 + c));
+      return ECC_S(ECC_P(0, 28, 21 + c), ECC_P(0, 27, 18 + c), ECC_P(0, 29, 24 + c));
     }
   }
 #undef ECC_S
@@ -97,8 +123,10 @@ __host__ __device__ bool view_geometry(FP P, FT th, bool moved, int W, int H, in
       const int r = k / 3, c = k % 3;
       const T sx = w.sc[0], cx = w.sc[1], sy = w.sc[2], cy = w.sc[3], sz = w.sc[4], cz = w.sc[5];
       const T x = r == 0 ? cz : sz;
-      const T a = r == 2 ? cy : x * sy, e = r == 0 ? -sz : (r == 1 ? cz : T(0.0));
-      w.R[k] = c == 0 ? (r == 2 ? -sy : x * cy) : (c == 1 ? a * sx + e * cx : a * cx - e * sx);
+      const T a = r == 2 ? cy : x * sy;  // column 1: a sx + e cx, column 2: a cx + e sx
+      const T e = r == 2 ? T(0.0) : (r == 0 ? (c == 1 ? -sz : sz) : (c == 1 ? cz : -cz));
+      const T f = c == 1 ? sx : cx, g = c == 1 ? cx : sx;
+      w.R[k] = c == 0 ? (r == 2 ? -sy : x * cy) : (k == 2 ? mad(e, g, a * f) : mad(a, f, e * g));
     }
     sync();
   }
@@ -106,7 +134,7 @@ __host__ __device__ bool view_geometry(FP P, FT th, bool moved, int W, int H, in
     if (moved) {
       const int i = k & ~3, j = k & 3;
       const T x = j < 3 ? w.R[j] : th(3), y = j < 3 ? w.R[3 + j] : th(4), z = j < 3 ? w.R[6 + j] : th(5);
-      const T s = P(i) * x + P(i + 1) * y + P(i + 2) * z;
+      const T s = mad(P(i + 2), z, mad(P(i), x, P(i + 1) * y));
       w.Pm[k] = j < 3 ? s : s + T(P(k));
     } else {
       w.Pm[k] = T(P(k));
@@ -123,7 +151,7 @@ __host__ __device__ bool view_geometry(FP P, FT th, bool moved, int W, int H, in
   const T* m3 = w.Pm + 8;
   const T det = m1[0] * (m2[1] * m3[2] - m2[2] * m3[1]) + m1[1] * (m2[2] * m3[0] - m2[0] * m3[2]) +
                 m1[2] * (m2[0] * m3[1] - m2[1] * m3[0]);
-  const T n3 = sqrt(m3[0] * m3[0] + m3[1] * m3[1] + m3[2] * m3[2]);
+  const T n3 = sqrt(mad(m3[2], m3[2], mad(m3[0], m3[0], m3[1] * m3[1])));
   bool ok = isfinite(value(det)) && isfinite(value(n3)) && value(det) != 0.0 && value(n3) > 0.0;
   for (int k = 0; k < 12; ++k) ok = ok && isfinite(value(w.Pm[k]));  // NaN / Inf anywhere, the motion's included
   const T sc = ok ? T(copysign(1.0, value(det))) / n3 : T(0.0);
@@ -134,7 +162,8 @@ __host__ __device__ bool view_geometry(FP P, FT th, bool moved, int W, int H, in
     const T* x = w.V + 4 * (m & 3);
     const T* y = w.V + 4 * (m >> 2 & 3);
     const int i = m >> 4 & 3, j = m >> 6;
-    w.V[12 + k] = x[i] * y[j] - x[j] * y[i];
+    // t and its copy in m1 x m2 with three roundings, as one shared difference of products
+    w.V[12 + k] = cross2(x[i], y[j], x[j], y[i], k != 4 && k != 13);
   }
   sync();
   for (int k = lane; k < 11; k += L) {
@@ -144,7 +173,7 @@ __host__ __device__ bool view_geometry(FP P, FT th, bool moved, int W, int H, in
       x[i] = w.V[m >> (11 * i + 5) & 31];
       if (m >> (11 * i + 10) & 1) x[i] = -x[i];
     }
-    w.S[k] = x[0] * w.V[m & 31] + x[1] * w.V[m >> 11 & 31] + x[2] * w.V[m >> 22 & 31];
+    w.S[k] = mad(x[2], w.V[m >> 22 & 31], mad(x[1], w.V[m >> 11 & 31], x[0] * w.V[m & 31]));
   }
   sync();
   ok = ok && value(w.S[3]) != 0.0;
@@ -153,7 +182,7 @@ __host__ __device__ bool view_geometry(FP P, FT th, bool moved, int W, int H, in
   ok = ok && value(nu) > 0.0;
   for (int k = lane; k < 15; k += L)
     w.q[k] = k < 3 ? w.S[k] * iw : (k < 6 ? (ok ? w.V[18 + k] / nu : T(0.0)) : (k < 12 ? w.V[12 + k] : w.S[k - 4]));
-  const T dd = w.S[6] - w.S[4] * w.S[4];
+  const T dd = mad(-w.S[4], w.S[4], w.S[6]);
   ok = ok && value(dd) > 0.0;
   const T D = ok ? sqrt(dd) : T(0.0);
   if (lane == 0) w.D = D;
@@ -265,6 +294,7 @@ struct GeometryRanges {
 };
 
 __global__ void __launch_bounds__(32) geometry_kernel(Geometry g, GeometryRanges n) {
+  let_next_start();
   __shared__ GeometryShared sh;
   int b = (int)blockIdx.x;
   if (b < n.views) {
@@ -714,10 +744,19 @@ __device__ void pair_grad_q(const PairRec& pr, const ViewRec* __restrict__ views
   }
 }
 
-__global__ void pair_grad_q_kernel(long long n_pairs, const PairRec* __restrict__ prs,
-                                   const ViewRec* __restrict__ views, const double* __restrict__ Gpp,
-                                   float2* __restrict__ gq) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// The first block sums the total meanwhile (a launch of its own before this one held up the
+// gradient by 8 us).
+__global__ void __launch_bounds__(kGradQThreads)
+    pair_grad_q_kernel(long long n_pairs, const PairRec* __restrict__ prs, const ViewRec* __restrict__ views,
+                       const double* __restrict__ Gpp, float2* __restrict__ gq, const double* __restrict__ partial,
+                       int n_partial, double* __restrict__ total) {
+  __shared__ double s[kSumSlots];
+  wait_for_previous();
+  if (blockIdx.x == 0) {
+    reduce_fixed<kGradQThreads>(partial, n_partial, total, s);
+    return;
+  }
+  const long long p = (long long)(blockIdx.x - 1) * kGradQThreads + threadIdx.x;
   if (p >= n_pairs) return;
   pair_grad_q(prs[p], views, Gpp + 12 * p, gq + 30 * p);
 }
@@ -754,13 +793,15 @@ __device__ void reduce_q_block(int lam, int n_views, long long n_pairs, const in
   }
   for (int k = 0; k < 15; ++k) sh[k][threadIdx.x] = make_float2(acc[k].hi, acc[k].lo);
   __syncthreads();
-  for (int wdt = blockDim.x / 2; wdt > 0; wdt >>= 1) {
-    if (threadIdx.x < wdt)
-      for (int k = 0; k < 15; ++k) {
-        const float2 x = sh[k][threadIdx.x], y = sh[k][threadIdx.x + wdt];
-        const df z = df_add(df{x.x, x.y}, df{y.x, y.y});
-        sh[k][threadIdx.x] = make_float2(z.hi, z.lo);
-      }
+  // a level's 15 wdt sums spread over all threads (by the first wdt threads alone the levels
+  // took 15 sums in a row each)
+  for (int wdt = 128; wdt > 0; wdt >>= 1) {
+    for (int i = threadIdx.x; i < 15 * wdt; i += 256) {
+      const int k = i / wdt, t = i % wdt;
+      const float2 x = sh[k][t], y = sh[k][t + wdt];
+      const df z = df_add(df{x.x, x.y}, df{y.x, y.y});
+      sh[k][t] = make_float2(z.hi, z.lo);
+    }
     __syncthreads();
   }
 }
@@ -785,6 +826,7 @@ __global__ void __launch_bounds__(256) view_grad_theta_kernel(int n_views, long 
                                                               const float2* __restrict__ gq,
                                                               const ViewTan* __restrict__ vtan,
                                                               double* __restrict__ grad) {
+  wait_for_previous();
   __shared__ float2 sh[15][256];
   const int lam = blockIdx.x;
   reduce_q_block(lam, n_views, n_pairs, pairs, gq, sh);
@@ -797,6 +839,7 @@ __global__ void __launch_bounds__(256) view_grad_P_kernel(int n_views, long long
                                                           const float2* __restrict__ gq,
                                                           const ViewTanP* __restrict__ vtan,
                                                           double* __restrict__ grad_P) {
+  wait_for_previous();
   __shared__ float2 sh[15][256];
   const int lam = blockIdx.x;
   reduce_q_block(lam, n_views, n_pairs, pairs, gq, sh);
@@ -829,7 +872,8 @@ __global__ void __launch_bounds__(32) serve_view_kernel(const ServeJob* __restri
   const ServeJob& J = jobs[j];
   if (!__any_sync(0xffffffffu, J.do_grad)) return;
   const long long v = i - voff[j];
-  device_tangent<false>(J.P + 12 * v, J.theta + 6 * v, dir, J.W, J.H, sh, J.do_grad && t < 6 * total, &J.vtan[v].dC[0][0]);
+  device_tangent<false>(J.P + 12 * v, J.theta + 6 * v, dir, J.W, J.H, sh, J.do_grad && t < 6 * total,
+                        &J.vtan[v].dC[0][0]);
 }
 
 __global__ void serve_pair_setup_kernel(const ServeJob* __restrict__ jobs, const long long* __restrict__ poff,

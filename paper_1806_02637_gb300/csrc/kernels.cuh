@@ -14,8 +14,9 @@ __global__ void pair_setup_kernel(int n_views, long long p_begin, long long p_en
                                   int reuse_sampling, int* status);
 __global__ void view_grad_theta_kernel(int n_views, long long n_pairs, const int32_t* pairs, const float2* gq,
                                        const ViewTan* vtan, double* grad);
+constexpr int kGradQThreads = 64;
 __global__ void pair_grad_q_kernel(long long n_pairs, const PairRec* prs, const ViewRec* views, const double* Gpp,
-                                   float2* gq);
+                                   float2* gq, const double* partial, int n_partial, double* total);
 __global__ void view_grad_P_kernel(int n_views, long long n_pairs, const int32_t* pairs, const float2* gq,
                                    const ViewTanP* vtan, double* grad_P);
 
@@ -64,6 +65,61 @@ struct LaunchHooks {
     if (end) end(ctx, n, s);
   }
 };
+
+// Kernels of a call that are launched behind the one before (programmatic dependent launch)
+// wait for its end and its stores as their first step: their launch and their blocks' start
+// overlap its end.  That takes 2 us to 5 us off a call of several short kernels (motion
+// gradient of 248 views 285 -> 282 us, evaluation of one pair 37.2 -> 35.0 us, two-view
+// precompute 43.8 -> 40.8 us).  Launched plainly: the first kernel of a call, which waits for
+// whatever the stream did before; pair_setup_kernel and ecc_pair_kernel, because an SM that
+// never falls idle between them keeps the first one's split of L1 and shared memory, at which
+// fewer blocks of the second fit (evaluation of the 496-view scan 567 -> 747 us).
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() {
+  let_next_start();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... K, class... A>
+void launch_at(bool behind, void (*kernel)(K...), dim3 grid, dim3 block, size_t shared, cudaStream_t stream,
+               A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = shared;
+  c.stream = stream;
+  c.attrs = &at;
+  c.numAttrs = behind ? 1 : 0;
+  cudaLaunchKernelEx(&c, kernel, K(args)...);  // the caller reads cudaGetLastError
+}
+template <class... K, class... A>
+void launch_behind(void (*kernel)(K...), dim3 grid, dim3 block, size_t shared, cudaStream_t stream, A... args) {
+  launch_at(true, kernel, grid, block, shared, stream, args...);
+}
+
+// Fixed-order sum of n block partials by one block of THREADS threads: as many chunks as
+// slots, one after the other, then a tree, whatever THREADS.
+constexpr int kSumSlots = 1024;
+template <int THREADS>
+__device__ __forceinline__ void reduce_fixed(const double* __restrict__ partial, int n, double* __restrict__ total,
+                                             double* s) {
+  const int per = (n + kSumSlots - 1) / kSumSlots;
+#pragma unroll 4
+  for (int t = threadIdx.x; t < kSumSlots; t += THREADS) {
+    double acc = 0.0;
+    const int end = min(n, (t + 1) * per);
+    for (int i = t * per; i < end; ++i) acc += partial[i];
+    s[t] = acc;
+  }
+  __syncthreads();
+  for (int w = kSumSlots / 2; w > 0; w >>= 1) {
+    for (int t = threadIdx.x; t < w; t += THREADS) s[t] += s[t + w];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *total = s[0];
+}
 
 // Parameters of the pair kernel for one scan (device pointers).
 struct PairArgs {
@@ -141,7 +197,8 @@ cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_a
                          const cudaEvent_t* batch_ready = nullptr);  // per batch: wait before reading its images
 cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n_views, const float* images, int W,
                                int H, int n_alpha, int n_s, void* planes, size_t plane_bytes, float* of,
-                               __nv_bfloat16* ob, int* status, const LaunchHooks& hooks, cudaStream_t stream);
+                               __nv_bfloat16* ob, int* status, bool behind, const LaunchHooks& hooks,
+                               cudaStream_t stream);
 
 cudaError_t launch_ecc_pairs(long long n_pairs, const PairRec* prs, const float4* ctile, int n_tiles,
                              const float4* alpha_dir, const void* sino, const float* scales, int dtype,

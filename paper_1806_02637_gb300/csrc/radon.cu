@@ -36,9 +36,11 @@ namespace {
 // [W][pitch_c] (pairs along y), the image from element pad on, zeros elsewhere
 // (the pair before the image carries (0, v[0])).  A block (32, 8) covers 32x32
 // pairs starting one pixel before the image; the weighted values of a 33x33 tile
-// are computed once into shared memory and both planes are written coalesced.
+// are computed once into shared memory and both planes are written coalesced.  The
+// blocks beside the margins write their zeros.
 __global__ void weight_kernel(const float* __restrict__ images, const RadonView* __restrict__ rv, int W, int H,
                               int pad, int pitch_r, int pitch_c, float2* __restrict__ wimg, size_t plane) {
+  wait_for_previous();
   __shared__ float tile[33][34];
   const int v = blockIdx.z;
   const float* g = images + (size_t)v * W * H;
@@ -67,6 +69,23 @@ __global__ void weight_kernel(const float* __restrict__ images, const RadonView*
     const int xo = bx + ty, yo = by + tx;
     if (xo >= 0 && xo < W && yo >= -1 && yo < H)
       T[(size_t)xo * pitch_c + yo + pad] = make_float2(tile[tx][ty], tile[tx + 1][ty] - tile[tx][ty]);
+  }
+  // margins: [0, pad - 1) before the image's pairs, [W + pad, W + 2 pad) behind them (H for columns)
+  const float2 zero = make_float2(0.0f, 0.0f);
+  for (int side = 0; side < 2; ++side) {
+    const int n = side ? pad : pad - 1;
+    if (blockIdx.x == (side ? gridDim.x - 1 : 0))
+      for (int j = threadIdx.y; j < 32; j += 8) {
+        const int y = by + j;
+        for (int i = threadIdx.x; y >= 0 && y < H && i < n; i += 32)
+          R[(size_t)y * pitch_r + (side ? W + pad : 0) + i] = zero;
+      }
+    if (blockIdx.y == (side ? gridDim.y - 1 : 0))
+      for (int j = threadIdx.y; j < 32; j += 8) {
+        const int x = bx + j;
+        for (int i = threadIdx.x; x >= 0 && x < W && i < n; i += 32)
+          T[(size_t)x * pitch_c + (side ? H + pad : 0) + i] = zero;
+      }
   }
 }
 
@@ -137,6 +156,7 @@ __global__ void __launch_bounds__(32 * kAlphaPerBlock) joseph_kernel(const Radon
                                                                       const float2* __restrict__ wimg, JosephArgs g,
                                                                       float* __restrict__ out_f32,
                                                                       __nv_bfloat16* __restrict__ out_bf16) {
+  wait_for_previous();
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   // the warps of a block take the same 31 outputs of consecutive alpha rows: their
@@ -216,6 +236,7 @@ __global__ void __launch_bounds__(32 * kAlphaPerBlock) joseph_kernel(const Radon
 // start at zero and scale_finalize_kernel turns them into scales in place.
 __global__ void __launch_bounds__(256) absmax_kernel(const float* __restrict__ s32, size_t per_view,
                                                      unsigned* __restrict__ max_bits) {
+  wait_for_previous();
   const float* __restrict__ p = s32 + (size_t)blockIdx.y * per_view;
   const size_t chunk = (per_view + gridDim.x - 1) / gridDim.x;
   const size_t beg = (size_t)blockIdx.x * chunk;
@@ -227,12 +248,14 @@ __global__ void __launch_bounds__(256) absmax_kernel(const float* __restrict__ s
 }
 
 __global__ void scale_finalize_kernel(float* __restrict__ scales, int n) {
+  wait_for_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) scales[i] = scales[i] > 0.0f ? scales[i] / 16384.0f : 1.0f;
 }
 
 __global__ void quantize_f16_kernel(const float* __restrict__ s32, size_t per_view, size_t n,
                                     const float* __restrict__ scales, __half* __restrict__ out) {
+  wait_for_previous();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   out[i] = __float2half_rn(s32[i] / scales[i / per_view]);
@@ -293,12 +316,12 @@ static cudaError_t quantize_batch(const float* stage, size_t per_view, int nb, f
   const unsigned per_block = 256 * 16;  // 16 elements per thread, at most 64 blocks per view
   const unsigned bpv = (unsigned)std::min<size_t>(64, (per_view + per_block - 1) / per_block);
   hooks.on_begin("absmax_kernel", stream);
-  absmax_kernel<<<dim3(bpv, nb), 256, 0, stream>>>(stage, per_view, reinterpret_cast<unsigned*>(scales));
+  launch_behind(absmax_kernel, dim3(bpv, nb), 256, 0, stream, stage, per_view, reinterpret_cast<unsigned*>(scales));
   hooks.on_end("absmax_kernel", stream);
-  scale_finalize_kernel<<<(nb + 255) / 256, 256, 0, stream>>>(scales, nb);
+  launch_behind(scale_finalize_kernel, (nb + 255) / 256, 256, 0, stream, scales, nb);
   const size_t n = per_view * nb;
   hooks.on_begin("quantize_f16_kernel", stream);
-  quantize_f16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(stage, per_view, n, scales, out);
+  launch_behind(quantize_f16_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, stage, per_view, n, scales, out);
   hooks.on_end("quantize_f16_kernel", stream);
   return cudaGetLastError();
 }
@@ -322,6 +345,7 @@ cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_a
   const int n_chunks = (n_s + 30) / 31;
   const size_t per_view = (size_t)n_alpha * n_s;
   float2* wv = reinterpret_cast<float2*>(wimg);
+  const bool behind = batch_ready == nullptr;  // behind an event a batch's first kernel is launched plainly
   for (int v0 = 0; v0 < n_views; v0 += plan.batch) {
     const int nb = min(plan.batch, n_views - v0);
     cudaError_t e;
@@ -331,17 +355,13 @@ cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_a
     float* of = dtype == 0 ? (float*)sino_out + oo : (dtype == 1 ? stage : nullptr);
     __nv_bfloat16* ob = dtype == 2 ? (__nv_bfloat16*)sino_out + oo : nullptr;
     if (plan.views) {
-      e = launch_radon_views(table, rv + v0, nb, im, W, H, n_alpha, n_s, wimg, plan.wimg_bytes, of, ob, status, hooks,
-                             stream);
+      e = launch_radon_views(table, rv + v0, nb, im, W, H, n_alpha, n_s, wimg, plan.wimg_bytes, of, ob, status, behind,
+                             hooks, stream);
       if (e != cudaSuccess) return e;
     } else {
-      if (v0 == 0) {  // zero margins; later batches overwrite only the pairs of the image
-        e = cudaMemsetAsync(wimg, 0, sizeof(float2) * jg.plane * nb, stream);
-        if (e != cudaSuccess) return e;
-      }
       hooks.on_begin("weight_kernel", stream);
-      weight_kernel<<<dim3((W + 32) / 32, (H + 32) / 32, nb), dim3(32, 8), 0, stream>>>(
-          im, rv + v0, W, H, jg.pad, jg.pitch_r, jg.pitch_c, wv, jg.plane);
+      launch_at(behind, weight_kernel, dim3((W + 32) / 32, (H + 32) / 32, nb), dim3(32, 8), 0, stream, im, rv + v0, W,
+                H, jg.pad, jg.pitch_r, jg.pitch_c, wv, jg.plane);
       hooks.on_end("weight_kernel", stream);
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
@@ -349,9 +369,9 @@ cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_a
       const dim3 grid(n_chunks, (n_alpha + kAlphaPerBlock - 1) / kAlphaPerBlock, nb), block(32 * kAlphaPerBlock);
       hooks.on_begin("joseph_kernel", stream);
       if (clamp)
-        joseph_kernel<true><<<grid, block, 0, stream>>>(tb, rv + v0, wv, jg, of, ob);
+        launch_behind(joseph_kernel<true>, grid, block, 0, stream, tb, rv + v0, wv, jg, of, ob);
       else
-        joseph_kernel<false><<<grid, block, 0, stream>>>(tb, rv + v0, wv, jg, of, ob);
+        launch_behind(joseph_kernel<false>, grid, block, 0, stream, tb, rv + v0, wv, jg, of, ob);
       hooks.on_end("joseph_kernel", stream);
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;

@@ -120,13 +120,14 @@ __device__ __forceinline__ void bulk_copy(unsigned dst, const void* src, unsigne
 // Weighted projections as differences along one axis or both, views innermost.  A block
 // takes 32 x 8 cells of the 32 views of a group: the weighted values of 33 x 9 pixels are
 // computed once into shared memory (reads coalesced along image rows) and the planes are
-// written in runs of 128 bytes.
+// written in runs of 128 bytes.  The blocks beside the margins write their zeros.
 constexpr int kTileX = 32, kTileY = 8;
 constexpr int kTilePitch = 33;
 
 __global__ void __launch_bounds__(256) weight_views_kernel(const float* __restrict__ images,
                                                            const RadonView* __restrict__ rv, ViewsArgs g,
                                                            float* __restrict__ planes) {
+  wait_for_previous();
   __shared__ float tile[(kTileX + 1) * (kTileY + 1) * kTilePitch];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int bx = (int)blockIdx.x * kTileX - 1, by = (int)blockIdx.y * kTileY - 1;
@@ -161,6 +162,11 @@ __global__ void __launch_bounds__(256) weight_views_kernel(const float* __restri
         rows[((size_t)y * pitch_r + x + 1 + g.pad) * kGroup + lane] = p[kTilePitch] - p[0];
       }
     }
+    const int y = by + 1 + warp;  // margins: a row per warp
+    if (y < g.H && blockIdx.x == 0)
+      for (int i = 0; i < g.pad; ++i) rows[((size_t)y * pitch_r + i) * kGroup + lane] = 0.0f;
+    if (y < g.H && blockIdx.x == gridDim.x - 1)
+      for (int i = 0; i < g.pad; ++i) rows[((size_t)y * pitch_r + g.W + 1 + g.pad + i) * kGroup + lane] = 0.0f;
   }
   if (g.axis != 0) {
     float* __restrict__ cols = planes + g.cols0 + (size_t)blockIdx.z * g.W * pitch_c * kGroup;
@@ -171,6 +177,13 @@ __global__ void __launch_bounds__(256) weight_views_kernel(const float* __restri
         const float* p = tile + (ty * (kTileX + 1) + tx) * kTilePitch + lane;
         cols[((size_t)x * pitch_c + y + 1 + g.pad) * kGroup + lane] = p[(kTileX + 1) * kTilePitch] - p[0];
       }
+    }
+    for (int t = warp; t < kTileX; t += 8) {
+      const int x = bx + 1 + t;
+      if (x < g.W && blockIdx.y == 0)
+        for (int i = 0; i < g.pad; ++i) cols[((size_t)x * pitch_c + i) * kGroup + lane] = 0.0f;
+      if (x < g.W && blockIdx.y == gridDim.y - 1)
+        for (int i = 0; i < g.pad; ++i) cols[((size_t)x * pitch_c + g.H + 1 + g.pad + i) * kGroup + lane] = 0.0f;
     }
   }
 }
@@ -287,6 +300,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
                                                                      float* __restrict__ out_f32,
                                                                      __nv_bfloat16* __restrict__ out_bf16,
                                                                      int* __restrict__ status) {
+  wait_for_previous();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) u64 bars[2 * kMaxSlots];
   __shared__ unsigned windows[kMaxSteps];   // of each step: start in the plane, cells << 16
@@ -564,7 +578,8 @@ int ViewsPlan::min_views(int W, int H, int n_alpha, int n_s) {
 
 cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n_views, const float* images, int W,
                                int H, int n_alpha, int n_s, void* scratch, size_t scratch_bytes, float* of,
-                               __nv_bfloat16* ob, int* status, const LaunchHooks& hooks, cudaStream_t stream) {
+                               __nv_bfloat16* ob, int* status, bool behind, const LaunchHooks& hooks,
+                               cudaStream_t stream) {
   const double s_max = spacing(W, H, n_s);
   ViewsArgs g{};
   g.W = W;
@@ -583,7 +598,7 @@ cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n
   cudaError_t e = cudaFuncSetAttribute(radon_views_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared);
   if (e != cudaSuccess) return e;
   const size_t grid = (size_t)n_alpha * n_s, px = (size_t)W * H;
-  const size_t pitch_r = (size_t)W + 1 + 2 * g.pad, pitch_c = (size_t)H + 1 + 2 * g.pad;
+  const size_t pitch_r = (size_t)W + 1 + 2 * g.pad;
   // the planes of both axes at once, or of one at a time where both do not fit
   const int axes = ViewsPlan::group_bytes(2, W, H, n_alpha, n_s) > scratch_bytes ? 1 : 2;
   const int fit = (int)std::min<size_t>(4096, scratch_bytes / ViewsPlan::group_bytes(axes, W, H, n_alpha, n_s));
@@ -594,31 +609,16 @@ cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n
     for (int pass = 0; pass < (axes == 2 ? 1 : 2); ++pass) {
       g.axis = axes == 2 ? 2 : pass;
       g.cols0 = g.axis == 2 ? (size_t)groups * H * pitch_r * kGroup : 0;
-      // zero cells beside the image
-      const size_t side = g.pad * (size_t)kCell;
-      if (g.axis != 1) {
-        e = cudaMemset2DAsync(planes, pitch_r * kCell, 0, side, (size_t)H * groups, stream);
-        if (e == cudaSuccess)
-          e = cudaMemset2DAsync(planes + (size_t)(W + 1 + g.pad) * kGroup, pitch_r * kCell, 0, side,
-                                (size_t)H * groups, stream);
-      }
-      if (g.axis != 0 && e == cudaSuccess) {
-        e = cudaMemset2DAsync(planes + g.cols0, pitch_c * kCell, 0, side, (size_t)W * groups, stream);
-        if (e == cudaSuccess)
-          e = cudaMemset2DAsync(planes + g.cols0 + (size_t)(H + 1 + g.pad) * kGroup, pitch_c * kCell, 0, side,
-                                (size_t)W * groups, stream);
-      }
-      if (e != cudaSuccess) return e;
       hooks.on_begin("weight_views_kernel", stream);
-      weight_views_kernel<<<dim3((W + kTileX) / kTileX, (H + kTileY) / kTileY, groups), 256, 0, stream>>>(
-          images + (size_t)v * px, rv + v, g, planes);
+      launch_at(behind, weight_views_kernel, dim3((W + kTileX) / kTileX, (H + kTileY) / kTileY, groups), 256, 0, stream,
+                images + (size_t)v * px, rv + v, g, planes);
       hooks.on_end("weight_views_kernel", stream);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       const int tiles = (g.axis != 1 ? t.rows : 0) + (g.axis != 0 ? t.cols : 0);
       if (tiles == 0) continue;
       hooks.on_begin("radon_views_kernel", stream);
-      radon_views_kernel<<<dim3(t.chunks, tiles, groups), 32 * kWarps, shared, stream>>>(
-          table, rv + v, planes, g, of ? of + (size_t)v * grid : nullptr, ob ? ob + (size_t)v * grid : nullptr, status);
+      launch_behind(radon_views_kernel, dim3(t.chunks, tiles, groups), 32 * kWarps, shared, stream, table, rv + v,
+                    planes, g, of ? of + (size_t)v * grid : nullptr, ob ? ob + (size_t)v * grid : nullptr, status);
       hooks.on_end("radon_views_kernel", stream);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
