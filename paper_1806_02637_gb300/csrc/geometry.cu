@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(32) geometry_kernel(Geometry g, GeometryRanges
       o.u0 = (float)w.u0();
       o.v0 = (float)w.v0();
       o.D = (float)w.D;
-      o.pad = 0;
+      o.max_bits = 0;
       g.weights[v] = o;
     }
     return;

@@ -32,7 +32,7 @@ struct RadonRow {
 
 struct RadonView {  // per-view weights (FP32 copies of the FP64 set-up)
   float u0, v0, D;
-  int pad;
+  unsigned max_bits;  // max |S| of a view staged for FP16, as bits
 };
 
 // The FP64 work of a call that depends on its geometry alone, in one launch: what is not
