@@ -62,6 +62,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = True):
     """Loads libecc.so (building it first if it is missing or stale)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -118,17 +120,30 @@ def load(build_if_missing: bool = True):
         return lib
 
 
+# A short call spends as long in Python as on the GPU (evaluation of one pair: 31 us to issue of
+# 35 us), so the marshalling below looks things up once, hands addresses to ctypes as plain
+# integers and does not check tensors that it has just allocated itself.
+_torch_mod = None
+_codes = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_mod
+    if _torch_mod is None:
+        import torch
+        _torch_mod = torch
+    return _torch_mod
 
 
 def _dtype_code(dt) -> int:
-    torch = _torch()
-    table = {torch.float32: ECC_F32, torch.float16: ECC_F16, torch.bfloat16: ECC_BF16}
-    if dt not in table:
+    global _codes
+    if _codes is None:
+        torch = _torch()
+        _codes = {torch.float32: ECC_F32, torch.float16: ECC_F16, torch.bfloat16: ECC_BF16}
+    code = _codes.get(dt)
+    if code is None:
         raise EccError(f"unsupported sinogram dtype {dt}")
-    return table[dt]
+    return code
 
 
 def _check(ctx, rc, what):
@@ -145,20 +160,23 @@ def _dev(t, dtype, name, shape=None):
         raise EccError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise EccError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise EccError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
     return t
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # without a Stream object around it
+    if raw is not None:
+        return raw(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 class Context:
@@ -237,14 +255,17 @@ def _eval_args(P, sino, motion, pairs, scales, total, per_pair, nkappa, want_per
     scales = _dev(scales, torch.float32, "scales", (N,)) if code == ECC_F16 else None
     if total is None:
         total = torch.empty((1,), dtype=torch.float64, device=dev)
-    _dev(total, torch.float64, "total", (1,))
+    else:
+        _dev(total, torch.float64, "total", (1,))
     if want_per_pair:
         if per_pair is None:
             per_pair = torch.empty((n_pairs, 2), dtype=torch.float64, device=dev)
+        else:
+            _dev(per_pair, torch.float64, "per_pair", (n_pairs, 2))
         if nkappa is None:
             nkappa = torch.empty((n_pairs,), dtype=torch.int32, device=dev)
-        _dev(per_pair, torch.float64, "per_pair", (n_pairs, 2))
-        _dev(nkappa, torch.int32, "nkappa", (n_pairs,))
+        else:
+            _dev(nkappa, torch.int32, "nkappa", (n_pairs,))
     return code, N, P, sino, motion, pairs, n_pairs, scales, total, per_pair, nkappa
 
 
@@ -330,7 +351,8 @@ def ecc_evaluate_grad(ctx: Context, P, sino, W: int, H: int, n_kappa: int, cauch
         P, sino, motion, pairs, scales, total, per_pair, nkappa, want_per_pair)
     if grad is None:
         grad = torch.empty((N, 6), dtype=torch.float64, device=sino.device)
-    _dev(grad, torch.float64, "grad", (N, 6))
+    else:
+        _dev(grad, torch.float64, "grad", (N, 6))
     rc = load().ecc_evaluate_grad(ctx.handle, N, _ptr(P), _ptr(motion), _ptr(sino), _ptr(scales), int(W), int(H),
                                   sino.shape[1], sino.shape[2], code, int(n_kappa), float(cauchy_c), _ptr(pairs),
                                   int(n_pairs), _ptr(total), _ptr(per_pair), _ptr(nkappa), _ptr(grad),
@@ -350,7 +372,8 @@ def ecc_evaluate_grad_projection(ctx: Context, P, sino, W: int, H: int, n_kappa:
         P, sino, motion, pairs, scales, total, per_pair, nkappa, want_per_pair)
     if grad_P is None:
         grad_P = torch.empty((N, 12), dtype=torch.float64, device=sino.device)
-    _dev(grad_P, torch.float64, "grad_P", (N, 12))
+    else:
+        _dev(grad_P, torch.float64, "grad_P", (N, 12))
     rc = load().ecc_evaluate_grad_projection(ctx.handle, N, _ptr(P), _ptr(motion), _ptr(sino), _ptr(scales),
                                              int(W), int(H), sino.shape[1], sino.shape[2], code, int(n_kappa),
                                              float(cauchy_c), _ptr(pairs), int(n_pairs), _ptr(total),
@@ -368,15 +391,16 @@ def _autograd_function():
         @staticmethod
         def forward(fctx, motion, ctx, P, sino, W, H, n_kappa, cauchy_c, pairs, scales):
             motion = motion.detach().contiguous()
+            total = torch.empty((), dtype=torch.float64, device=sino.device)
             if motion.requires_grad or fctx.needs_input_grad[0]:
                 r = ecc_evaluate_grad(ctx, P, sino, W, H, n_kappa, cauchy_c, motion=motion, pairs=pairs,
-                                      scales=scales, want_per_pair=False)
+                                      scales=scales, total=total.view(1), want_per_pair=False)
                 fctx.save_for_backward(r["grad"])
             else:
-                r = ecc_evaluate(ctx, P, sino, W, H, n_kappa, cauchy_c, motion=motion, pairs=pairs, scales=scales,
-                                 want_per_pair=False)
+                ecc_evaluate(ctx, P, sino, W, H, n_kappa, cauchy_c, motion=motion, pairs=pairs, scales=scales,
+                             total=total.view(1), want_per_pair=False)
                 fctx.save_for_backward(torch.zeros_like(motion))
-            return r["total"][0].clone()
+            return total
 
         @staticmethod
         def backward(fctx, g):
