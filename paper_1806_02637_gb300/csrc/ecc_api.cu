@@ -277,12 +277,9 @@ int run_evaluate(ecc_ctx* c, int n_views, const double* P, const double* motion,
   // One pair set-up launch, then one pair-kernel launch, on the caller's stream.  (Set-up
   // chunks on a second stream beside the pair kernel's chunks were measured slower: the
   // two kernels sharing SMs slowed each other, 0.707 -> 0.765 ms on the 496-view scan.)
-  hk.on_begin("pair_setup_kernel", s);
-  ecc::pair_setup_kernel<<<(unsigned)((np + 127) / 128), 128, 0, s>>>(
-      n_views, 0, np, pairs, (const ecc::ViewRec*)c->views.p, W, H, n_kappa, (ecc::PairRec*)c->pairs.p,
-      (float4*)c->ctile.p, n_tiles, reuse ? 1 : 0, c->d_status);
-  hk.on_end("pair_setup_kernel", s);
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "pair set-up launch");
+  e = ecc::launch_pair_setup(n_views, np, pairs, (const ecc::ViewRec*)c->views.p, W, H, n_kappa,
+                             (ecc::PairRec*)c->pairs.p, (float4*)c->ctile.p, n_tiles, reuse, c->d_status, hk, s);
+  if (e != cudaSuccess) return cuda_fail(c, e, "pair set-up launch");
   int nb = 0;
   e = ecc::launch_ecc_pairs(np, (const ecc::PairRec*)c->pairs.p, (const float4*)c->ctile.p, n_tiles,
                             (const float4*)c->adir.p, sino, scales, dtype, n_alpha, n_s, n_kappa, W, H, cauchy_c,

@@ -134,9 +134,8 @@ extern "C" int ecc_evaluate_noalloc(int n_views, const double* P, const double* 
   g.n_alpha = n_alpha;
   g.alpha_dir = adir;
   if ((e = ecc::launch_geometry(g, hk, s)) != cudaSuccess) return fail(ECC_ECUDA, cudaGetErrorString(e));
-  ecc::pair_setup_kernel<<<(n_pairs + 127) / 128, 128, 0, s>>>(n_views, 0, n_pairs, pairs, views, W, H, n_kappa, prs,
-                                                               ctile, n_tiles, 0, status);
-  if ((e = cudaGetLastError()) != cudaSuccess) return fail(ECC_ECUDA, cudaGetErrorString(e));
+  e = ecc::launch_pair_setup(n_views, n_pairs, pairs, views, W, H, n_kappa, prs, ctile, n_tiles, false, status, hk, s);
+  if (e != cudaSuccess) return fail(ECC_ECUDA, cudaGetErrorString(e));
   int nb = 0;
   e = ecc::launch_ecc_pairs(n_pairs, prs, ctile, n_tiles, adir, sino, scales, dtype, n_alpha, n_s, n_kappa, W, H,
                             cauchy_c, per_pair, nkappa, partial, nullptr, status, &nb, hk, s);

@@ -534,8 +534,13 @@ __host__ __device__ __noinline__ df view_arc(const df* A, int W, int H, df* clo)
 // double-float copies: the frame, the maps, the corner values and signs, the angles
 // (df_atan2, df_sincos), the step and the positions whose floors give the integer
 // ranges.
+//
+// LANES = 2: lanes 2 i and 2 i + 1 of a warp (side 0, 1; the whole warp calls) take one
+// view's map and arc each, which go to r.Af[0], and the same steps otherwise; each writes
+// every other tile direction.  The values are the same.
+template <int LANES>
 __host__ __device__ PairRec setup_pair(int a, int b, int n_views, const ViewRec* views, int W, int H, int K,
-                                       float4* ctile, int n_tiles, const PairRec* previous) {
+                                       float4* ctile, int n_tiles, const PairRec* previous, int side = 0) {
   const bool reuse_sampling = previous != nullptr;
   PairRec r;
   const bool in_range = a >= 0 && b >= 0 && a < n_views && b < n_views;
@@ -555,23 +560,39 @@ __host__ __device__ PairRec setup_pair(int a, int b, int n_views, const ViewRec*
   r.c0[1] = 0.0;
   const ViewRec& va = views[a];
   const ViewRec& vb = views[b];
+  constexpr int kSides = LANES == 1 ? 2 : 1;  // of this lane
   df w[3], v[3];
-  df Ad[2][6];
+  df Ad[kSides][6];
+  df len[2] = {}, cl[2][2] = {};
   bool ok = in_range && va.status == 0 && vb.status == 0 && a != b && pencil_frame_df(va, vb, w, v);
   if (ok) {
-    const ViewRec* vv[2] = {&va, &vb};
-    for (int s = 0; s < 2; ++s)
+    const ViewRec* vv[2] = {LANES == 1 || side == 0 ? &va : &vb, &vb};
+    for (int s = 0; s < kSides; ++s)
       for (int i = 0; i < 3; ++i) {
         const df row[3] = {qget(*vv[s], 6 + 3 * i), qget(*vv[s], 7 + 3 * i), qget(*vv[s], 8 + 3 * i)};
         Ad[s][2 * i + 0] = df_dot3(row, w);
         Ad[s][2 * i + 1] = df_dot3(row, v);
       }
-    for (int s = 0; s < 2; ++s)
+    for (int s = 0; s < kSides; ++s)
       for (int i = 0; i < 6; ++i) {
         r.Af[s][2 * i] = Ad[s][i].hi;
         r.Af[s][2 * i + 1] = Ad[s][i].lo;
       }
+    if (!reuse_sampling)
+      for (int s = 0; s < kSides; ++s) len[s] = view_arc(Ad[s], W, H, cl[s]);
   }
+#ifdef __CUDA_ARCH__
+  if (LANES == 2) {
+    auto other = [](df x) { return df{__shfl_xor_sync(0xffffffffu, x.hi, 1), __shfl_xor_sync(0xffffffffu, x.lo, 1)}; };
+    const df lo = other(len[0]), xo = other(cl[0][0]), yo = other(cl[0][1]);
+    len[1] = df_sel(side == 0, lo, len[0]);
+    cl[1][0] = df_sel(side == 0, xo, cl[0][0]);
+    cl[1][1] = df_sel(side == 0, yo, cl[0][1]);
+    len[0] = df_sel(side == 0, len[0], lo);
+    cl[0][0] = df_sel(side == 0, cl[0][0], xo);
+    cl[0][1] = df_sel(side == 0, cl[0][1], yo);
+  }
+#endif
   if (ok && reuse_sampling) {
     // keep the planes sampled by the previous call (kappa arcs and validity
     // frozen); only the kappa -> line maps follow the new geometry
@@ -588,15 +609,13 @@ __host__ __device__ PairRec setup_pair(int a, int b, int n_views, const ViewRec*
     r.nk = old.nk;
     ok = old.status == 0;
   } else if (ok) {
-    df cla[2], clb[2];
-    const df lena = view_arc(Ad[0], W, H, cla);
-    const df lenb = view_arc(Ad[1], W, H, clb);
+    const df lena = len[0], lenb = len[1];
     // sample the shorter arc; ties (equal in exact arithmetic for mirror-symmetric
     // pairs) go to view a within a relative tolerance, not by rounding
     const bool samp_a = df_sub(lena, lenb).hi <= 1e-9f * fmaxf(lena.hi, lenb.hi);
     const df len_s = samp_a ? lena : lenb, len_o = samp_a ? lenb : lena;
-    const df csx = samp_a ? cla[0] : clb[0], csy = samp_a ? cla[1] : clb[1];
-    const df cox = samp_a ? clb[0] : cla[0], coy = samp_a ? clb[1] : cla[1];
+    const df csx = samp_a ? cl[0][0] : cl[1][0], csy = samp_a ? cl[0][1] : cl[1][1];
+    const df cox = samp_a ? cl[1][0] : cl[0][0], coy = samp_a ? cl[1][1] : cl[0][1];
     const df dk = df_div_f(len_s, (float)K);
     r.dk = df_to_double(dk);
     r.dk_hi = dk.hi;
@@ -659,7 +678,8 @@ __host__ __device__ PairRec setup_pair(int a, int b, int n_views, const ViewRec*
     rotate(c16, s16, csx, csy, &cx0, &cy0);
     float4* ct = ctile;
     for (int t = 0; t < n_tiles; ++t) {
-      if (32 * t + 32 <= K) {
+      if (LANES == 2 && (t & 1) != side) {
+      } else if (32 * t + 32 <= K) {
         ct[t] = make_float4(cx0.hi, cy0.hi, cx0.lo, cy0.lo);
       } else {  // last, partial tile
         df sp, cp, px, py;
@@ -677,12 +697,16 @@ __host__ __device__ PairRec setup_pair(int a, int b, int n_views, const ViewRec*
   return r;
 }
 
-__global__ void pair_setup_kernel(int n_views, long long p_begin, long long p_end, const int32_t* __restrict__ pairs,
+// One thread per pair, or two.
+template <int LANES>
+__global__ void pair_setup_kernel(int n_views, long long n_pairs, const int32_t* __restrict__ pairs,
                                   const ViewRec* __restrict__ views, int W, int H, int K,
                                   PairRec* __restrict__ out, float4* __restrict__ ctile, int n_tiles,
                                   int reuse_sampling, int* __restrict__ status) {
-  const long long p = p_begin + (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= p_end) return;
+  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+  if (LANES == 1 && i >= n_pairs) return;
+  const long long p = i < n_pairs ? i : n_pairs - 1;  // LANES = 2: the warp stays whole
+  const int side = LANES == 1 ? 0 : threadIdx.x & 1;
   int a, b;
   if (pairs) {
     a = pairs[2 * p];
@@ -692,10 +716,56 @@ __global__ void pair_setup_kernel(int n_views, long long p_begin, long long p_en
   }
   PairRec prev;
   if (reuse_sampling) prev = out[p];
-  const PairRec r = setup_pair(a, b, n_views, views, W, H, K, ctile + p * n_tiles, n_tiles,
-                               reuse_sampling ? &prev : nullptr);
-  if (r.status) atomicOr(status, kStatusDegeneratePair);
-  out[p] = r;
+  if (LANES == 2) __syncwarp();  // both have read it
+  PairRec r = setup_pair<LANES>(a, b, n_views, views, W, H, K, ctile + p * n_tiles, n_tiles,
+                                reuse_sampling ? &prev : nullptr, side);
+  if (LANES == 1) {
+    if (r.status) atomicOr(status, kStatusDegeneratePair);
+    out[p] = r;
+    return;
+  }
+  if (i >= n_pairs) return;
+  PairRec& o = out[p];
+  for (int k = 0; k < 12; ++k) o.Af[side][k] = r.Af[0][k];
+  if (side == 0) {
+    if (r.status) atomicOr(status, kStatusDegeneratePair);
+    o.dk_hi = r.dk_hi;
+    o.dk_lo = r.dk_lo;
+    o.c0[0] = r.c0[0];
+    o.c0[1] = r.c0[1];
+    o.dk = r.dk;
+    o.a = r.a;
+    o.b = r.b;
+    o.r0lo = r.r0lo;
+    o.r0hi = r.r0hi;
+    o.r1lo = r.r1lo;
+    o.r1hi = r.r1hi;
+    o.nk = r.nk;
+    o.status = r.status;
+  }
+}
+
+// Two threads per pair while that leaves a scheduler with one warp: a pair's steps wait on
+// each other, and the second thread takes one view's map and arc off the first (evaluation of
+// one pair 35.2 -> 33.8 us, of a list without allocation 55.7 -> 53.3 us, gradient of 7140
+// pairs 107.0 -> 104.7 us).  With more pairs the instructions bound the kernel, and two
+// threads execute more of them than one.
+cudaError_t launch_pair_setup(int n_views, long long n_pairs, const int32_t* pairs, const ViewRec* views, int W, int H,
+                              int K, PairRec* out, float4* ctile, int n_tiles, bool reuse_sampling, int* status,
+                              const LaunchHooks& hooks, cudaStream_t stream) {
+  int dev = 0, n_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  hooks.on_begin("pair_setup_kernel", stream);
+  if (2 * n_pairs <= 4 * 32 * (long long)n_sm)
+    pair_setup_kernel<2><<<(unsigned)((2 * n_pairs + 63) / 64), 64, 0, stream>>>(
+        n_views, n_pairs, pairs, views, W, H, K, out, ctile, n_tiles, reuse_sampling, status);
+  else
+    pair_setup_kernel<1><<<(unsigned)((n_pairs + 127) / 128), 128, 0, stream>>>(
+        n_views, n_pairs, pairs, views, W, H, K, out, ctile, n_tiles, reuse_sampling, status);
+  hooks.on_end("pair_setup_kernel", stream);
+  return cudaGetLastError();
 }
 
 // Gradient of one pair's e with respect to the per-view quantities the pair reads,
@@ -885,7 +955,7 @@ __global__ void serve_pair_setup_kernel(const ServeJob* __restrict__ jobs, const
   const long long p = i - poff[j];
   int a, b;
   pair_from_index(p, J.n_views, &a, &b);
-  const PairRec r = setup_pair(a, b, J.n_views, J.views, J.W, J.H, J.pair.K,
+  const PairRec r = setup_pair<1>(a, b, J.n_views, J.views, J.W, J.H, J.pair.K,
                                const_cast<float4*>(J.pair.ctile) + p * J.n_tiles, J.n_tiles, nullptr);
   if (r.status) atomicOr(J.status, kStatusDegeneratePair);
   const_cast<PairRec*>(J.pair.prs)[p] = r;
@@ -1026,7 +1096,7 @@ extern "C" int ecc_internal_setup_pair_host(int n_views, const double* P, const 
   }
   const int n_tiles = (K + 31) / 32;
   float4* ct = new float4[n_tiles];
-  const ecc::PairRec r = ecc::setup_pair(0, 1, 2, views, W, H, K, ct, n_tiles, nullptr);
+  const ecc::PairRec r = ecc::setup_pair<1>(0, 1, 2, views, W, H, K, ct, n_tiles, nullptr);
   delete[] ct;
   info_out[0] = r.c0[0];
   info_out[1] = r.c0[1];

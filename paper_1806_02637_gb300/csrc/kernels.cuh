@@ -9,9 +9,6 @@
 namespace ecc {
 
 // pairs [p_begin, p_end) of the row-major a < b enumeration (pairs == NULL) or of the list
-__global__ void pair_setup_kernel(int n_views, long long p_begin, long long p_end, const int32_t* pairs,
-                                  const ViewRec* views, int W, int H, int K, PairRec* out, float4* ctile, int n_tiles,
-                                  int reuse_sampling, int* status);
 __global__ void view_grad_theta_kernel(int n_views, long long n_pairs, const int32_t* pairs, const float2* gq,
                                        const ViewTan* vtan, double* grad);
 constexpr int kGradQThreads = 64;
@@ -191,6 +188,9 @@ struct ViewsPlan {
 
 // Launchers (return cudaError_t of the launch).
 cudaError_t launch_geometry(const Geometry& g, const LaunchHooks& hooks, cudaStream_t stream);
+cudaError_t launch_pair_setup(int n_views, long long n_pairs, const int32_t* pairs, const ViewRec* views, int W, int H,
+                              int K, PairRec* out, float4* ctile, int n_tiles, bool reuse_sampling, int* status,
+                              const LaunchHooks& hooks, cudaStream_t stream);
 cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_alpha, int n_s, int dtype,
                          void* sino_out, float* scales_out, const RadonRow* table, void* wimg, float* stage,
                          const RadonPlan& plan, int* status, const LaunchHooks& hooks, cudaStream_t stream,
