@@ -150,12 +150,18 @@ __device__ __forceinline__ void joseph_block(const float2* __restrict__ rp, floa
   }
 }
 
+// Three blocks per SM (80 registers): the kernel waits on its loads, and with registers to
+// spare the compiler issues 16 rows' loads together.  Left to itself it takes 64 (a view of
+// 256 x 256 on the 256 x 363 grid 28.5 us, now 20.4; 12 views of 620 x 480 1.296 ms, now
+// 1.268; a 976 x 976 view 450 us, now 435); two blocks are 1 % faster on many views and 3 %
+// slower on two.  (Several warps along one line, and the next rows' loads issued before these
+// rows' sums, did not pay: 31 us stayed 31 us for two views, more views got slower.)
 template <bool CLAMP>
-__global__ void __launch_bounds__(32 * kAlphaPerBlock) joseph_kernel(const RadonRow* __restrict__ table,
-                                                                      const RadonView* __restrict__ rv,
-                                                                      const float2* __restrict__ wimg, JosephArgs g,
-                                                                      float* __restrict__ out_f32,
-                                                                      __nv_bfloat16* __restrict__ out_bf16) {
+__global__ void __launch_bounds__(32 * kAlphaPerBlock, 3) joseph_kernel(const RadonRow* __restrict__ table,
+                                                                         const RadonView* __restrict__ rv,
+                                                                         const float2* __restrict__ wimg,
+                                                                         JosephArgs g, float* __restrict__ out_f32,
+                                                                         __nv_bfloat16* __restrict__ out_bf16) {
   wait_for_previous();
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
