@@ -767,27 +767,33 @@ def run_ours(args):
     dom = max(prof.items(), key=lambda kv: kv[1][1])[0]
     peaks = measured_peaks()
     n_dom, ms_dom = prof[dom]
-    if dom == "joseph_kernel":
+    if dom in ("joseph_kernel", "radon_views_kernel"):
         taps = joseph_taps(cfg)
         flops = FLOPS_PER_TAP * taps * args.steps / n_dom
         achieved = flops / (ms_dom / n_dom / 1e3) / 1e12
-        # DRAM bytes (read + write) of one launch, from an ncu capture of a 32-view launch of this
-        # kernel (183.3 MB + 58.3 MB), scaled to the views of an average launch of this step
+        # DRAM bytes (read + write) of one launch, from ncu captures (joseph_kernel: 32 views, 183.3 MB +
+        # 58.3 MB; radon_views_kernel: 128 views, 400.7 MB + 276.1 MB), scaled to the views of an average
+        # launch of this step
         views_per_launch = cfg.n_views * args.steps / n_dom
-        traffic = (183.299840e6 + 58.299392e6) / 32 * views_per_launch
+        captured, per_view = ((32, (183.299840e6 + 58.299392e6) / 32) if dom == "joseph_kernel" else
+                              (128, (400.717056e6 + 276.057088e6) / 128))
         roof = {"kernel": dom, "bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved / FP32_PEAK_TFLOPS, "traffic": traffic,
-                "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of a 32-view launch, "
+                "frac": achieved / FP32_PEAK_TFLOPS, "traffic": per_view * views_per_launch,
+                "traffic_source": f"ncu dram__bytes_read.sum + dram__bytes_write.sum of a {captured}-view launch, "
                                   f"scaled to {views_per_launch:.1f} views per launch",
                 "peak_source": "FP32 lanes x FMA x max SM clock (152 x 128 x 2 x 2.07 GHz)",
-                "work": f"{FLOPS_PER_TAP} FLOP per in-image Joseph tap, {taps} taps per step",
-                # the kernel's actual limiter (ncu: L1 data-pipe wavefronts): the 8-byte
-                # interpolation pair each tap reads, against the L1 data rate
-                "l1_gather": {"achieved_tbs": 8.0 * taps * args.steps / n_dom / (ms_dom / n_dom / 1e3) / 1e12,
-                              "peak_tbs": L1_PEAK_TBS,
-                              "frac": 8.0 * taps * args.steps / n_dom / (ms_dom / n_dom / 1e3) / 1e12 / L1_PEAK_TBS,
-                              "peak_source": "128 B per clock per SM x 152 SMs x 2.07 GHz",
-                              "work": "8 B (one interpolation pair) per in-image tap"}}
+                "work": f"{FLOPS_PER_TAP} FLOP per in-image Joseph tap, {taps} taps per step"}
+        if dom == "joseph_kernel":
+            # the kernel's actual limiter (ncu: L1 data-pipe wavefronts): the 8-byte
+            # interpolation pair each tap reads, against the L1 data rate
+            tbs = 8.0 * taps * args.steps / n_dom / (ms_dom / n_dom / 1e3) / 1e12
+            roof["l1_gather"] = {"achieved_tbs": tbs, "peak_tbs": L1_PEAK_TBS, "frac": tbs / L1_PEAK_TBS,
+                                 "peak_source": "128 B per clock per SM x 152 SMs x 2.07 GHz",
+                                 "work": "8 B (one interpolation pair) per in-image tap"}
+        else:
+            # one walk along a line serves 32 views: no single limiter (ncu, 128 views)
+            roof["limits"] = {"issue": 0.67, "shared_memory_reads": 0.68, "fma_pipes": 0.54,
+                              "source": "ncu, 128 views of 620 x 480 on the 768 x 768 grid, of each peak"}
     else:
         bytes_per_launch = 32.0 * units * args.steps / n_dom
         achieved = bytes_per_launch / (ms_dom / n_dom / 1e3) / 1e9

@@ -20,11 +20,11 @@
 // Work split: a lane follows 16 lines of one alpha row for four views; a warp holds four
 // neighbouring alpha rows x 32 views.  Where the four rows' lines are in one cell, the
 // warp's 16-byte loads fall into the same 128 bytes of shared memory, which are read once
-// (3.2 wavefronts a load instead of 4 on the 620 x 480 grid).  A CTA takes 16 warps = A neighbouring alpha rows x 64 / A
-// neighbouring chunks of 16 lines.  Their lines cross one image step within a window of
-// some dozen cells; each step's window (contiguous in memory) is brought into a ring of
-// shared-memory slots by one bulk asynchronous copy, which the warps issue in turn some
-// steps ahead.  The 64 accumulators of a lane stay in registers.
+// (3.2 wavefronts a load instead of 4 on the 620 x 480 grid).  A CTA takes 16 warps = A
+// neighbouring alpha rows x 64 / A neighbouring chunks of 16 lines.  Their lines cross one
+// image step within a window of some dozen cells; each step's window (contiguous in memory)
+// is brought into a ring of shared-memory slots by one bulk asynchronous copy, which the
+// warps issue in turn some steps ahead.  The 64 accumulators of a lane stay in registers.
 //
 // Measured on 128 views of 620 x 480, 768 x 768 grid: 5.60 ms (view by view: 14.5).  No one
 // resource bounds it: issue 67 %, shared-memory reads 68 %, FMA pipes 54 % of their peaks.
@@ -474,7 +474,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
   for (int i = 0; i < kLines; ++i)
 #pragma unroll
     for (int e = 0; e < 4; ++e)
-      mine[(sub * kGroup + vl * 4 + e) * kPitch + (rev ? kLines - 1 - i : i)] = (e == 0 ? acc[i].x : e == 1 ? acc[i].y : e == 2 ? acc[i].z : acc[i].w) * norm;
+      mine[(sub * kGroup + vl * 4 + e) * kPitch + (rev ? kLines - 1 - i : i)] =
+          (e == 0 ? acc[i].x : e == 1 ? acc[i].y : e == 2 ? acc[i].z : acc[i].w) * norm;
   __syncwarp();
   const int vbase = (int)blockIdx.z * kGroup;
   for (int a = 0; a < kRows; ++a) {
