@@ -565,16 +565,22 @@ static Tiles tiles_of(int W, int H, int n_alpha, int n_s) {
   return t;
 }
 
-// A group takes as long as about 13 views of the view-by-view form where its CTAs fill the
-// GPU for some waves (one group against 12 and 14 views, in us: 1,716 against 1,351 and
-// 1,603 on 620 x 480, 6,050 against 5,316 and 6,188 on 976 x 976), and longer in proportion
-// where they do not (256 x 256, 102 CTAs: 330 with 32 views against 358, 465 with 64 against
-// 740).  A rule on the sizes alone: two waves of a GPU of 152 SMs.
+// A group takes as long as about 15 views of the view-by-view form where its CTAs fill the
+// GPU for some waves (one group against 15 and 16 views, in us: 1,701 against 1,644 and
+// 1,756 on 620 x 480, 6,030 against 6,349 and 6,790 on 976 x 976), and longer in proportion
+// where they do not: on 256 x 256 (102 CTAs a group) two groups take 412 against 389 for 39
+// views, on 300 x 260 (221 CTAs) one takes 479 against 440 for 20 and 486 against 546 for 25.
+// Where lines are closer together than a cell (more work per line, and windows with more
+// lines) it takes up to half as long again (97 views of 18 x 126, ds = 0.46: 139 against 93);
+// there from the second group on, whose last views may be few.  A rule on the sizes alone, at
+// which the many-view form was the faster one on ten grids: two waves of a GPU of 152 SMs.
 int ViewsPlan::min_views(int W, int H, int n_alpha, int n_s) {
   const Tiles t = tiles_of(W, H, n_alpha, n_s);
   if (t.A == 0) return 0;
   const double ctas = (double)(t.rows + t.cols) * t.chunks;
-  return (int)std::ceil(13.0 * std::max(1.0, 304.0 / ctas));
+  const bool close = std::sqrt((double)W * W + (double)H * H) / (n_s - 1) < 0.99;
+  const double least = std::max(close ? 48.0 : 16.0, 16.0 * 304.0 / ctas * (close ? 1.5 : 1.0));
+  return (int)std::ceil(least);
 }
 
 cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n_views, const float* images, int W,

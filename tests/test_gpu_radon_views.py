@@ -34,13 +34,13 @@ def _precompute(P, images, n_alpha, n_s, dtype=torch.float32, budget=0):
 
 # the bar of the FP32 precompute (max|dS| <= 1e-5 max|S| per view)
 @pytest.mark.parametrize("n,W,Hh,n_alpha,n_s", [
-    (25, 300, 260, 512, 400),   # one group, partly filled
-    (290, 97, 61, 90, 113),     # nine groups and two views
-    (256, 40, 100, 61, 200),    # line spacing 0.54 .. 0.77 cells: two lines in one cell
-    (150, 101, 33, 256, 78),    # line spacing 1.38 .. 1.95 cells
-    (287, 31, 30, 160, 44),     # image narrower than a chunk of lines
-    (321, 48, 47, 96, 67),      # line spacing 1.00 .. 1.44 cells
-    (97, 18, 126, 101, 276),    # eight alpha rows per block
+    (26, 300, 260, 512, 400),   # one group, partly filled
+    (354, 97, 61, 90, 113),     # eleven groups and two views
+    (460, 40, 100, 61, 200),    # line spacing 0.54 .. 0.77 cells: two lines in one cell
+    (185, 101, 33, 256, 78),    # line spacing 1.38 .. 1.95 cells
+    (351, 31, 30, 160, 44),     # image narrower than a chunk of lines
+    (353, 48, 47, 96, 67),      # line spacing 1.00 .. 1.44 cells
+    (168, 18, 126, 101, 276),   # eight alpha rows per block
 ])
 def test_many_views_against_oracle(n, W, Hh, n_alpha, n_s):
     P, images = _scan(n, W, Hh, 1000 * n + W)
