@@ -39,6 +39,7 @@ struct ecc_ctx {
   int device = 0;
   size_t budget = 0;
   size_t held = 0;
+  unsigned long long wait_ns = ecc::kWaitNs;  // limit of the precompute's device waits
   std::string err;
   int* d_status = nullptr;
   Buf views, pairs, ctile, adir, perpair, nk, partial, rtable, wimg, stage;
@@ -176,6 +177,7 @@ int ensure_precompute(ecc_ctx* c, int n_views, int W, int H, int n_alpha, int n_
   size_t cap = kViewsScratch;
   for (;;) {
     *plan = ecc::radon_plan(n_views, W, H, n_alpha, n_s, dtype, max_batch, cap, 0);
+    plan->wait_ns = c->wait_ns;
     rc = ensure(c, c->rtable, plan->table_bytes(n_views, n_alpha), "radon table");
     if (rc == ECC_OK) rc = ensure(c, c->wimg, plan->wimg_bytes, "weighted images");
     if (rc == ECC_OK && plan->stage_bytes) rc = ensure(c, c->stage, plan->stage_bytes, "FP16 staging");
@@ -666,6 +668,14 @@ extern "C" int ecc_internal_dump(ecc_ctx* c, void* stream, int n_views, int n_pa
   if (e == cudaSuccess && n_pairs > 0 && pairs_out && c->pairs.p)
     e = cudaMemcpy(pairs_out, c->pairs.p, sizeof(ecc::PairRec) * (size_t)n_pairs, cudaMemcpyDeviceToHost);
   return e == cudaSuccess ? ECC_OK : cuda_fail(c, e, "dump");
+}
+
+// Internal (tests only): the limit of the context's bounded device waits in nanoseconds.
+// With 0 a wait gives up unless its first tries succeed.
+extern "C" int ecc_internal_set_wait_ns(ecc_ctx* c, unsigned long long ns) {
+  if (!c) return ECC_EINVAL;
+  c->wait_ns = ns;
+  return ECC_OK;
 }
 
 extern "C" int ecc_internal_record_sizes(int* view_bytes, int* pair_bytes) {

@@ -158,7 +158,9 @@ inline void pair_args_grid(PairArgs& g, int n_alpha, int n_s, int W, int H) {
 // (radon_views.cu), others view by view (radon.cu).  The choice between the two
 // depends on the sizes alone, and the many-view sums do not depend on how the views are
 // grouped, so that a scan's sinograms are the same wherever they are computed.
+constexpr unsigned long long kWaitNs = 1000000000ull;  // a bounded device wait gives up after this long
 struct RadonPlan {
+  unsigned long long wait_ns = kWaitNs;
   bool views;          // many views at once
   int batch;           // views per pass over the scratch
   size_t wimg_bytes;   // weighted images
@@ -197,8 +199,8 @@ cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_a
                          const cudaEvent_t* batch_ready = nullptr);  // per batch: wait before reading its images
 cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n_views, const float* images, int W,
                                int H, int n_alpha, int n_s, void* planes, size_t plane_bytes, float* of,
-                               __nv_bfloat16* ob, int* status, bool behind, const LaunchHooks& hooks,
-                               cudaStream_t stream);
+                               __nv_bfloat16* ob, int* status, unsigned long long wait_ns, bool behind,
+                               const LaunchHooks& hooks, cudaStream_t stream);
 
 cudaError_t launch_ecc_pairs(long long n_pairs, const PairRec* prs, const float4* ctile, int n_tiles,
                              const float4* alpha_dir, const void* sino, const float* scales, int dtype,

@@ -406,8 +406,8 @@ cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_a
     float* of = dtype == 0 ? (float*)sino_out + oo : (dtype == 1 ? stage : nullptr);
     __nv_bfloat16* ob = dtype == 2 ? (__nv_bfloat16*)sino_out + oo : nullptr;
     if (plan.views) {
-      e = launch_radon_views(table, rv + v0, nb, im, W, H, n_alpha, n_s, wimg, plan.wimg_bytes, of, ob, status, behind,
-                             hooks, stream);
+      e = launch_radon_views(table, rv + v0, nb, im, W, H, n_alpha, n_s, wimg, plan.wimg_bytes, of, ob, status, plan.wait_ns,
+                             behind, hooks, stream);
       if (e != cudaSuccess) return e;
     } else {
       hooks.on_begin("weight_kernel", stream);

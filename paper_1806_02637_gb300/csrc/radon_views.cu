@@ -52,7 +52,7 @@ constexpr int kRing = 190 * 1024; // shared memory of the slots
 constexpr int kMinSlots = 4;
 constexpr int kMaxSlots = 16;
 constexpr int kMaxSteps = 2048;   // of the window table
-constexpr unsigned long long kWaitNs = 1000000000ull;  // a wait gives up after this long
+constexpr unsigned kAll = 0xffffffffu;  // lanes of a warp
 
 struct ViewsArgs {
   int W, H, n_alpha, n_s;
@@ -64,6 +64,8 @@ struct ViewsArgs {
   int win;                 // most cells of a window
   size_t cols0;            // floats from the row planes to the column planes
   float ds;
+  unsigned long long wait_ns;  // a wait gives up after this long
+  unsigned hint;           // longest suspension of one of its tries, in ns
 };
 
 typedef unsigned long long u64;
@@ -81,31 +83,48 @@ __device__ __forceinline__ void mbar_expect(unsigned bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
 }
-// One try, in which the hardware may suspend the warp for up to 20 us (polling without the
-// hint took 35 instructions a step).
-__device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, %3;\n"
-      " selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(20000u)
-      : "memory");
-  return ok != 0;
-}
 __device__ __forceinline__ u64 now_ns() {
   u64 t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
 }
-// Waits for the phase of `parity` to complete; false if it, or another wait of the CTA,
-// gave up.
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatile int* failed) {
-  if (mbar_try(bar, parity)) return true;
+// One try, in which the hardware may suspend the warp for up to `hint` ns (polling without
+// the hint took 35 instructions a step).
+__device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity, unsigned hint) {
+  unsigned ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, %3;\n"
+      " selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(hint)
+      : "memory");
+  return ok != 0;
+}
+// Waits for the phase of `parity` to complete, by one thread; false if that took longer than
+// the limit, or if a wait of the CTA has given up meanwhile (failed, or NULL).
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, u64 limit_ns, unsigned hint,
+                                          volatile int* failed) {
+  if (mbar_try(bar, parity, hint)) return true;
   const u64 t0 = now_ns();
-  do {
-    if (mbar_try(bar, parity)) return true;
-  } while (now_ns() - t0 < kWaitNs && !*failed);
+  for (;;) {
+    const bool out = now_ns() - t0 >= limit_ns || (failed && *failed);
+    if (mbar_try(bar, parity, hint)) return true;
+    if (out) break;
+  }
+  if (failed) *failed = 1;
+  return false;
+}
+// The same by a whole warp, with one verdict for all lanes: lanes that disagreed would part,
+// some to the next step's warp barriers and some to the CTA's, and wait there for each other.
+__device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned parity, u64 limit_ns, unsigned hint,
+                                               volatile int* failed) {
+  if (__all_sync(kAll, mbar_try(bar, parity, hint))) return true;
+  const u64 t0 = now_ns();
+  for (;;) {
+    const bool out = now_ns() - t0 >= limit_ns || *failed;
+    if (__all_sync(kAll, mbar_try(bar, parity, hint))) return true;
+    if (__any_sync(kAll, out)) break;
+  }
   *failed = 1;
   return false;
 }
@@ -307,6 +326,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
   __shared__ int range[kWarps][2];          // steps of each warp
   __shared__ longlong2 line[kUnits];        // first line of each unit at step 0, advance per step
   __shared__ long long span[kUnits];        // from its first line to its last
+  __shared__ int armed[kMaxSlots];          // parity of the last phase a slot's copies were issued in, -1: none
   __shared__ int failed, widest;
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
   const int sub = lane >> 3, vl = lane & 7;
@@ -357,6 +377,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
   if (threadIdx.x == 0) {
     failed = widest = 0;
     for (int i = 0; i < kMaxSlots; ++i) {
+      armed[i] = -1;
       mbar_init(bar0 + 8 * i, 1);
       mbar_init(bar0 + 8 * (kMaxSlots + i), kWarps);
     }
@@ -396,15 +417,16 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
   const int slots = min(kMaxSlots, (int)((unsigned)kRing / slot_bytes));
   const unsigned slot0 = smem_u32(smem);
   bool ok = true;
-  // one lane: copies the window of step n into its slot
-  auto refill = [&](int n, int slot) {
+  // one lane: copies the window of step n into its slot, whose phase has this parity
+  auto refill = [&](int n, int slot, int parity) {
     const unsigned w = windows[n], bytes = (w >> 16) * kCell, bar = bar0 + 8 * slot;
+    armed[slot] = parity;
     mbar_expect(bar, bytes);
     if (bytes)
       bulk_copy(slot0 + slot * slot_bytes, plane + ((size_t)(j_lo + n) * pitch + (w & 0xffffu)) * kGroup, bytes, bar);
   };
   if (lane == 0)
-    for (int n = warp; n < min(slots, n_steps); n += kWarps) refill(n, n);
+    for (int n = warp; n < min(slots, n_steps); n += kWarps) refill(n, n, 0);
   __syncwarp();
 
   float4 acc[kLines];
@@ -422,8 +444,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
     for (int n = 0; n < n_steps; ++n, window_at += 4) {
       if (n >= kLag) {
         if ((n & (kWarps - 1)) == warp && n - kLag + slots < n_steps) {
-          if (lane == 0 && mbar_wait(bar0 + 8 * (kMaxSlots + slot_r), turn_r, &failed))
-            refill(n - kLag + slots, slot_r);
+          if (lane == 0 && mbar_wait(bar0 + 8 * (kMaxSlots + slot_r), turn_r, g.wait_ns, g.hint, &failed))
+            refill(n - kLag + slots, slot_r, turn_r ^ 1);
           __syncwarp();
         }
         if (++slot_r == slots) {
@@ -431,8 +453,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
           turn_r ^= 1;
         }
       }
-      ok = mbar_wait(full, turn, &failed);
-      if (!ok) break;
+      ok = mbar_wait_warp(full, turn, g.wait_ns, g.hint, &failed);
+      if (!ok) break;  // warp-uniform
       if (n >= n_lo && n < n_hi) {
         // exact position of the first line, FP32 steps for the lines after it
         unsigned window;
@@ -457,15 +479,15 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
     walk(std::true_type{});
   else
     walk(std::false_type{});
-  // a wait that gave up is reported; the copies in flight are waited for before the shared
-  // memory is given back
-  if (!ok || failed) {
-    if (lane == 0) atomicOr(status, kStatusTimeout);
-    int never = 0;
-    for (int i = 0; i < min(slots, n_steps); ++i)
-      for (int p = 0; p < 2; ++p) mbar_wait(bar0 + 8 * i, p, &never);
+  // A wait that gave up is reported.  No warp issues copies any more; those in flight land
+  // before the shared memory is given back.
+  if (__syncthreads_or(!ok || failed)) {
+    if (threadIdx.x < kMaxSlots && armed[threadIdx.x] >= 0)
+      mbar_wait(bar0 + 8 * threadIdx.x, (unsigned)armed[threadIdx.x], kWaitNs, g.hint, nullptr);
+    if (threadIdx.x == 0) atomicOr(status, kStatusTimeout);
+    __syncthreads();
+    return;
   }
-  if (__syncthreads_or(!ok || failed)) return;
   // transpose through shared memory: [alpha row][view][line], then runs of 16 outputs
   constexpr int kPitch = kLines + 1;
   float* __restrict__ mine = reinterpret_cast<float*>(smem) + warp * (kRows * kGroup * kPitch);
@@ -585,7 +607,7 @@ int ViewsPlan::min_views(int W, int H, int n_alpha, int n_s) {
 
 cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n_views, const float* images, int W,
                                int H, int n_alpha, int n_s, void* scratch, size_t scratch_bytes, float* of,
-                               __nv_bfloat16* ob, int* status, bool behind, const LaunchHooks& hooks,
+                               __nv_bfloat16* ob, int* status, u64 wait_ns, bool behind, const LaunchHooks& hooks,
                                cudaStream_t stream) {
   const double s_max = spacing(W, H, n_s);
   ViewsArgs g{};
@@ -594,6 +616,8 @@ cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n
   g.n_alpha = n_alpha;
   g.n_s = n_s;
   g.ds = (float)(std::sqrt((double)W * W + (double)H * H) / (n_s - 1));
+  g.wait_ns = wait_ns;
+  g.hint = (unsigned)std::min<u64>(wait_ns, 20000);
   const Tiles t = tiles_of(W, H, n_alpha, n_s);
   g.A = t.A;
   g.r1 = t.r1;
