@@ -15,7 +15,9 @@
 //                        there is at most one cell in between, so a line costs one load
 //                        (1.15 with the cells in between, averaged over the angles) and
 //                        two FMAs, and the half-step difference of Eq. 1 is accumulated
-//                        directly: no difference of two large sums is ever taken.
+//                        directly: no difference of two large sums is ever taken.  Every
+//                        line's position is exact (32.32 fixed point), and the sums of
+//                        32 steps are folded into a second level in tensor memory.
 //
 // Work split: a lane follows 16 lines of one alpha row for four views; a warp holds four
 // neighbouring alpha rows x 32 views.  Where the four rows' lines are in one cell, the
@@ -26,8 +28,9 @@
 // is brought into a ring of shared-memory slots by one bulk asynchronous copy, which the
 // warps issue in turn some steps ahead.  The 64 accumulators of a lane stay in registers.
 //
-// Measured on 128 views of 620 x 480, 768 x 768 grid: 5.60 ms (view by view: 14.5).  No one
-// resource bounds it: issue 67 %, shared-memory reads 68 %, FMA pipes 54 % of their peaks.
+// Measured on 496 views of 620 x 480, 768 x 768 grid, the whole precompute: 23.5 ms (view by
+// view: 56.0; lines stepped in FP32 and sums of one level, which are less accurate than
+// view by view on noise: 22.3).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -240,77 +243,142 @@ __device__ __forceinline__ void fma4(float4& o, float w, const float4& d) {
   o = make_float4(a.x, a.y, b.x, b.y);
 }
 
-// Lines I and I + 1 of a lane at one step.  b + I cells: the cell after line I - 1's, f its
-// fraction.  Where the position moves by two cells (predicates p, q) the cell in between
-// goes to the output as it is; m holds it (registers that only some lanes write would stay
-// live around the loop if they were not kept across steps).  Loads and predicated sums of
-// both lines first, then their FMAs, so that no two neighbouring instructions depend on one
-// another.  NEAR: positions may also stay in their cell (predicate r), which the output then
-// holds once too often.
+// Weights of a position with fraction n / 2^32: f of the cell it is in, g = 1 - f.
+__device__ __forceinline__ float frac_f(unsigned n) { return __uint2float_rn(n) * 0x1p-32f; }
+__device__ __forceinline__ float frac_g(unsigned n) { return fmaf(__uint2float_rn(n), -0x1p-32f, 1.0f); }
+
+// Lines I and I + 1 of a lane at one step.  b + I cells: the cell after line I - 1's, n the
+// fraction of its position.  A line is s = 1 + step / 2^32 cells after the one before, so
+// that a carry out of the fractions' sum means a move by two cells (predicates p, q): the
+// cell in between goes to the output as it is; m holds it (registers that only some lanes
+// write would stay live around the loop if they were not kept across steps).  Loads and
+// predicated sums of both lines first, then their FMAs, so that no two neighbouring
+// instructions depend on one another.  NEAR: lanes with `below` set have s = step / 2^32,
+// and no carry means that the position stays in its cell (predicates r, t): the output is
+// then (f1 - f) d, of which the line before has put in (1 - f) d.
 template <bool NEAR, int I>
-__device__ __forceinline__ void two_lines(unsigned& b, float& f, float s1, float4& d, float4 (&m)[2],
+__device__ __forceinline__ void two_lines(unsigned& b, unsigned& n, unsigned step, bool below, float4 (&m)[2],
                                           float4 (&acc)[kLines]) {
-  float f1, f2;
+  unsigned n1, n2;
   float4 d1, d2;
   float4 &o = acc[I - 1], &o2 = acc[I];
+  float w1, w2;
   if (NEAR) {
+    unsigned stay1, stay2;
     asm volatile(
-        "{\n .reg .pred p, q, r, s;\n"
-        " add.f32 %0, %27, %28;\n"
-        " setp.lt.f32 r, %0, 0f00000000;\n @r add.f32 %0, %0, 0f3f800000;\n @r sub.u32 %2, %2, 128;\n"
-        " @r sub.f32 %3, %3, %29;\n @r sub.f32 %4, %4, %30;\n @r sub.f32 %5, %5, %31;\n @r sub.f32 %6, %6, %32;\n"
-        " setp.ge.f32 p, %0, 0f3f800000;\n @p ld.shared.v4.f32 {%11, %12, %13, %14}, [%2 + %33];\n"
-        " @p add.f32 %0, %0, 0fbf800000;\n @p add.u32 %2, %2, 128;\n"
-        " ld.shared.v4.f32 {%19, %20, %21, %22}, [%2 + %33];\n"
-        " add.f32 %1, %0, %28;\n"
-        " setp.lt.f32 s, %1, 0f00000000;\n @s add.f32 %1, %1, 0f3f800000;\n @s sub.u32 %2, %2, 128;\n"
-        " setp.ge.f32 q, %1, 0f3f800000;\n @q ld.shared.v4.f32 {%15, %16, %17, %18}, [%2 + %34];\n"
-        " @q add.f32 %1, %1, 0fbf800000;\n @q add.u32 %2, %2, 128;\n"
-        " ld.shared.v4.f32 {%23, %24, %25, %26}, [%2 + %34];\n"
+        "{\n .reg .pred p, q, r, t, u;\n"
+        " setp.ne.u32 u, %31, 0;\n"
+        " add.u32 %0, %29, %30;\n"
+        " setp.ge.and.u32 r, %0, %29, u;\n @r sub.u32 %2, %2, 128;\n"
+        " setp.lt.and.u32 p, %0, %29, !u;\n @p ld.shared.v4.f32 {%11, %12, %13, %14}, [%2 + %32];\n"
+        " @p add.u32 %2, %2, 128;\n"
+        " ld.shared.v4.f32 {%19, %20, %21, %22}, [%2 + %32];\n"
+        " add.u32 %1, %0, %30;\n"
+        " setp.ge.and.u32 t, %1, %0, u;\n @t sub.u32 %2, %2, 128;\n"
+        " setp.lt.and.u32 q, %1, %0, !u;\n @q ld.shared.v4.f32 {%15, %16, %17, %18}, [%2 + %33];\n"
+        " @q add.u32 %2, %2, 128;\n"
+        " ld.shared.v4.f32 {%23, %24, %25, %26}, [%2 + %33];\n"
+        " selp.u32 %27, 1, 0, r;\n selp.u32 %28, 1, 0, t;\n"
         " @p add.f32 %3, %3, %11;\n @p add.f32 %4, %4, %12;\n @p add.f32 %5, %5, %13;\n @p add.f32 %6, %6, %14;\n"
-        " @s sub.f32 %7, %7, %19;\n @s sub.f32 %8, %8, %20;\n @s sub.f32 %9, %9, %21;\n @s sub.f32 %10, %10, %22;\n"
         " @q add.f32 %7, %7, %15;\n @q add.f32 %8, %8, %16;\n @q add.f32 %9, %9, %17;\n @q add.f32 %10, %10, %18;\n}"
-        : "=&f"(f1), "=&f"(f2), "+r"(b), "+f"(o.x), "+f"(o.y), "+f"(o.z), "+f"(o.w), "+f"(o2.x), "+f"(o2.y),
+        : "=&r"(n1), "=&r"(n2), "+r"(b), "+f"(o.x), "+f"(o.y), "+f"(o.z), "+f"(o.w), "+f"(o2.x), "+f"(o2.y),
           "+f"(o2.z), "+f"(o2.w), "+f"(m[0].x), "+f"(m[0].y), "+f"(m[0].z), "+f"(m[0].w), "+f"(m[1].x), "+f"(m[1].y),
           "+f"(m[1].z), "+f"(m[1].w), "=&f"(d1.x), "=&f"(d1.y), "=&f"(d1.z), "=&f"(d1.w), "=&f"(d2.x), "=&f"(d2.y),
-          "=&f"(d2.z), "=&f"(d2.w)
-        : "f"(f), "f"(s1), "f"(d.x), "f"(d.y), "f"(d.z), "f"(d.w), "n"(I * 128), "n"(I * 128 + 128));
+          "=&f"(d2.z), "=&f"(d2.w), "=&r"(stay1), "=&r"(stay2)
+        : "r"(n), "r"(step), "r"((unsigned)below), "n"(I * 128), "n"(I * 128 + 128));
+    w1 = stay1 ? -frac_g(n1) : frac_f(n1);
+    w2 = stay2 ? -frac_g(n2) : frac_f(n2);
   } else {
     asm volatile(
         "{\n .reg .pred p, q;\n"
-        " add.f32 %0, %27, %28;\n"
-        " setp.ge.f32 p, %0, 0f3f800000;\n @p ld.shared.v4.f32 {%11, %12, %13, %14}, [%2 + %29];\n"
-        " @p add.f32 %0, %0, 0fbf800000;\n @p add.u32 %2, %2, 128;\n"
+        " add.u32 %0, %27, %28;\n"
+        " setp.lt.u32 p, %0, %27;\n @p ld.shared.v4.f32 {%11, %12, %13, %14}, [%2 + %29];\n"
+        " @p add.u32 %2, %2, 128;\n"
         " ld.shared.v4.f32 {%19, %20, %21, %22}, [%2 + %29];\n"
-        " add.f32 %1, %0, %28;\n"
-        " setp.ge.f32 q, %1, 0f3f800000;\n @q ld.shared.v4.f32 {%15, %16, %17, %18}, [%2 + %30];\n"
-        " @q add.f32 %1, %1, 0fbf800000;\n @q add.u32 %2, %2, 128;\n"
+        " add.u32 %1, %0, %28;\n"
+        " setp.lt.u32 q, %1, %0;\n @q ld.shared.v4.f32 {%15, %16, %17, %18}, [%2 + %30];\n"
+        " @q add.u32 %2, %2, 128;\n"
         " ld.shared.v4.f32 {%23, %24, %25, %26}, [%2 + %30];\n"
         " @p add.f32 %3, %3, %11;\n @p add.f32 %4, %4, %12;\n @p add.f32 %5, %5, %13;\n @p add.f32 %6, %6, %14;\n"
         " @q add.f32 %7, %7, %15;\n @q add.f32 %8, %8, %16;\n @q add.f32 %9, %9, %17;\n @q add.f32 %10, %10, %18;\n}"
-        : "=&f"(f1), "=&f"(f2), "+r"(b), "+f"(o.x), "+f"(o.y), "+f"(o.z), "+f"(o.w), "+f"(o2.x), "+f"(o2.y),
+        : "=&r"(n1), "=&r"(n2), "+r"(b), "+f"(o.x), "+f"(o.y), "+f"(o.z), "+f"(o.w), "+f"(o2.x), "+f"(o2.y),
           "+f"(o2.z), "+f"(o2.w), "+f"(m[0].x), "+f"(m[0].y), "+f"(m[0].z), "+f"(m[0].w), "+f"(m[1].x), "+f"(m[1].y),
           "+f"(m[1].z), "+f"(m[1].w), "=&f"(d1.x), "=&f"(d1.y), "=&f"(d1.z), "=&f"(d1.w), "=&f"(d2.x), "=&f"(d2.y),
           "=&f"(d2.z), "=&f"(d2.w)
-        : "f"(f), "f"(s1), "n"(I * 128), "n"(I * 128 + 128));
+        : "r"(n), "r"(step), "n"(I * 128), "n"(I * 128 + 128));
+    w1 = frac_f(n1);
+    w2 = frac_f(n2);
   }
-  fma4(o, f1, d1);
-  fma4(o2, f2, d2);
-  fma4(o2, 1.0f - f1, d1);
-  if constexpr (I + 1 < kLines) fma4(acc[I + 1], 1.0f - f2, d2);
-  f = f2;
-  d = d2;
-  if constexpr (I + 2 < kLines) two_lines<NEAR, I + 2>(b, f, s1, d, m, acc);
+  fma4(o, w1, d1);
+  fma4(o2, w2, d2);
+  fma4(o2, frac_g(n1), d1);
+  if constexpr (I + 1 < kLines) fma4(acc[I + 1], frac_g(n2), d2);
+  n = n2;
+  if constexpr (I + 2 < kLines) two_lines<NEAR, I + 2>(b, n, step, below, m, acc);
 }
 
-// One step of a lane's lines: the first at cell address b and fraction f, each next one
-// s = 1 + s1 cells further.  NEAR: some line spacing of the warp is below one cell, so
-// that two lines may share a cell.
+// One step of a lane's lines: the first at cell address b and fraction n, each next one
+// `step` further (its fraction; 1 + step / 2^32 cells, or without the 1 where `below`).
+// NEAR: some line spacing of the warp is below one cell, so that two lines may share a cell.
 template <bool NEAR>
-__device__ __forceinline__ void walk_step(unsigned b, float f, float s1, float4 (&m)[2], float4 (&acc)[kLines]) {
-  float4 d = load4(b);
-  fma4(acc[0], 1.0f - f, d);
-  two_lines<NEAR, 1>(b, f, s1, d, m, acc);
+__device__ __forceinline__ void walk_step(unsigned b, unsigned n, unsigned step, bool below, float4 (&m)[2],
+                                          float4 (&acc)[kLines]) {
+  fma4(acc[0], frac_g(n), load4(b));
+  two_lines<NEAR, 1>(b, n, step, below, m, acc);
+}
+
+// Second level of the sums, in tensor memory (a lane's 64 accumulators take all its
+// registers, the ring all shared memory): every kFold steps the accumulators are added to
+// it and keep what the addition rounds off, which the next fold takes along.  Rounding then
+// grows with the kFold steps of a block instead of all of up to 2048.  Error over max|S|
+// against 64 bits, in a restatement on the CPU over 40 grids of 160 to 976 pixels: of white
+// noise at most 0.57 times that of the view-by-view form (one level, lines stepped in FP32:
+// 3.7), of smooth images 0.26 times (1.5).  Blocks of 16 steps: 0.51 and 0.14.
+constexpr int kFold = 32;
+constexpr unsigned kTmemCols = 64 * kWarps / 4;  // a warp owns 32 lanes and 64 columns
+
+// Where a warp's part starts: its 32 lanes in the upper half of the address, its columns below.
+__device__ __forceinline__ unsigned tmem_of(unsigned base, int warp) {
+  return base + ((unsigned)(warp & 3) << 21) + 64u * (unsigned)(warp >> 2);
+}
+// Eight columns of the lane's second level (more at a time would spill).  The wait belongs
+// to the load: the registers are not valid before it.
+__device__ __forceinline__ void tmem_load(unsigned at, float4 (&v)[2]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+      " tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[0].z), "=f"(v[0].w), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[1].z), "=f"(v[1].w)
+      : "r"(at)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_store(unsigned at, const float4 (&v)[2]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"f"(v[0].x),
+               "f"(v[0].y), "f"(v[0].z), "f"(v[0].w), "f"(v[1].x), "f"(v[1].y), "f"(v[1].z), "f"(v[1].w), "r"(at)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_stored() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// s += y, y = what that rounds off.
+__device__ __forceinline__ void fold1(float& s, float& y) {
+  const float t = s + y;
+  y = y - (t - s);
+  s = t;
+}
+__device__ __forceinline__ void fold(unsigned at, float4 (&acc)[kLines]) {
+#pragma unroll
+  for (int c = 0; c < kLines / 2; ++c) {
+    float4 s[2];
+    tmem_load(at + 8 * c, s);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      float4& y = acc[2 * c + i];
+      fold1(s[i].x, y.x);
+      fold1(s[i].y, y.y);
+      fold1(s[i].z, y.z);
+      fold1(s[i].w, y.w);
+    }
+    tmem_store(at + 8 * c, s);
+  }
+  tmem_stored();
 }
 
 __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const RadonRow* __restrict__ table,
@@ -328,6 +396,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
   __shared__ long long span[kUnits];        // from its first line to its last
   __shared__ int armed[kMaxSlots];          // parity of the last phase a slot's copies were issued in, -1: none
   __shared__ int failed, widest;
+  __shared__ unsigned tmem_base;
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
   const int sub = lane >> 3, vl = lane & 7;
   // alpha rows of the tile: tiles of the two segments stepping over rows, then of the columns
@@ -349,7 +418,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
   // lines in the order of increasing position: k0 .. k0 + 16, or back where the step is negative
   const bool rev = row.STEP < 0;
   const long long step_q = rev ? -row.STEP : row.STEP;
-  const float s1 = (float)((double)(step_q - (1ll << 32)) * (1.0 / 4294967296.0));
+  const unsigned step = (unsigned)step_q;      // fraction of the line spacing
+  const bool below = step_q < (1ll << 32);     // the spacing is below one cell (and below two always)
   const long long first = row.B0 + (long long)(rev ? k0 + kLines : k0) * row.STEP;  // at step 0
   int lo_w = 0, hi_w = 0;
   if (live) {
@@ -363,7 +433,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
     hi_w = __reduce_max_sync(0xffffffffu, some ? hi_w : 0);
     if (hi_w < lo_w) hi_w = lo_w;
   }
-  const bool near = __any_sync(0xffffffffu, step_q < (1ll << 32) + 4096);
+  const bool near = __any_sync(0xffffffffu, below);
   const unsigned bar0 = smem_u32(bars);
   if (lane == 0) {
     range[warp][0] = lo_w;
@@ -383,7 +453,15 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 0) {  // the only CTA of its SM (shared memory), so that the columns are free
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                 "n"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  }
   __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   int j_lo = steps, j_hi = 0;
   for (int w = 0; w < kWarps; ++w)
     if (range[w][1] > range[w][0]) {
@@ -433,6 +511,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
 #pragma unroll
   for (int i = 0; i < kLines; ++i) acc[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   float4 m[2] = {acc[0], acc[0]};
+  for (int c = 0; c < kLines / 2; ++c) tmem_store(tmem_of(tmem_base, warp) + 8 * c, m);  // zeros
+  tmem_stored();
   auto walk = [&](auto near_lines) {
     long long X = first + (long long)lo_w * row.DY;
     const int n_lo = lo_w - j_lo, n_hi = hi_w - j_lo;
@@ -456,13 +536,13 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
       ok = mbar_wait_warp(full, turn, g.wait_ns, g.hint, &failed);
       if (!ok) break;  // warp-uniform
       if (n >= n_lo && n < n_hi) {
-        // exact position of the first line, FP32 steps for the lines after it
+        // exact positions of all lines: whole cells and a 32-bit fraction
         unsigned window;
         asm volatile("ld.shared.u16 %0, [%1];" : "=r"(window) : "r"(window_at));
         const unsigned b = slot_at + (unsigned)((int)(X >> 32) - (int)window) * kCell;
-        const float f0 = __uint_as_float(0x3f800000u | ((unsigned)X >> 9)) - 1.0f;
-        walk_step<decltype(near_lines)::value>(b, f0, s1, m, acc);
+        walk_step<decltype(near_lines)::value>(b, (unsigned)X, step, below, m, acc);
         X += row.DY;
+        if (((n - n_lo) & (kFold - 1)) == kFold - 1) fold(tmem_of(tmem_base, warp), acc);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(full + 8 * kMaxSlots);
@@ -479,9 +559,26 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
     walk(std::true_type{});
   else
     walk(std::false_type{});
+  // each accumulator and its second level together
+#pragma unroll
+  for (int c = 0; c < kLines / 2; ++c) {
+    float4 s[2];
+    tmem_load(tmem_of(tmem_base, warp) + 8 * c, s);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      float4& a = acc[2 * c + i];
+      a = make_float4(s[i].x + a.x, s[i].y + a.y, s[i].z + a.z, s[i].w + a.w);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   // A wait that gave up is reported.  No warp issues copies any more; those in flight land
   // before the shared memory is given back.
-  if (__syncthreads_or(!ok || failed)) {
+  const bool gave_up = __syncthreads_or(!ok || failed);
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols) : "memory");
+  }
+  if (gave_up) {
     if (threadIdx.x < kMaxSlots && armed[threadIdx.x] >= 0)
       mbar_wait(bar0 + 8 * threadIdx.x, (unsigned)armed[threadIdx.x], kWaitNs, g.hint, nullptr);
     if (threadIdx.x == 0) atomicOr(status, kStatusTimeout);
