@@ -40,6 +40,7 @@ struct ecc_ctx {
   size_t budget = 0;
   size_t held = 0;
   unsigned long long wait_ns = ecc::kWaitNs;  // limit of the precompute's device waits
+  size_t device_limit = 0;                    // tests: allocations beyond it fail as on a full device
   std::string err;
   int* d_status = nullptr;
   Buf views, pairs, ctile, adir, perpair, nk, partial, rtable, wimg, stage;
@@ -75,7 +76,26 @@ int cuda_fail(ecc_ctx* c, cudaError_t e, const char* what) {
   return fail(c, ECC_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
-// Grow-only scratch allocation, bounded by the context budget.
+void drop(ecc_ctx* c, Buf& b) {
+  if (!b.p) return;
+  cudaFree(b.p);  // synchronises the device: no kernel still uses the buffer
+  c->held -= b.n;
+  b = Buf{};
+}
+
+// The large buffers of the precompute, which no other call reads.
+void drop_precompute(ecc_ctx* c) {
+  drop(c, c->wimg);
+  drop(c, c->stage);
+}
+
+cudaError_t scratch_alloc(ecc_ctx* c, Buf& b, size_t bytes) {
+  if (c->device_limit && c->held + bytes > c->device_limit) return cudaErrorMemoryAllocation;
+  return cudaMalloc(&b.p, bytes);
+}
+
+// Grow-only scratch allocation, bounded by the context budget.  A context without a budget
+// gives the precompute's buffers back before it fails for want of device memory.
 int ensure(ecc_ctx* c, Buf& b, size_t bytes, const char* name) {
   if (bytes == 0) bytes = 16;
   if (b.n >= bytes) return ECC_OK;
@@ -83,13 +103,13 @@ int ensure(ecc_ctx* c, Buf& b, size_t bytes, const char* name) {
   if (c->budget && c->held - old + bytes > c->budget)
     return fail(c, ECC_ENOMEM, "scratch '%s' of %zu bytes exceeds the context budget (%zu held of %zu)", name, bytes,
                 c->held, c->budget);
-  if (b.p) {
-    cudaFree(b.p);  // synchronises the device: no kernel still uses the old buffer
-    b.p = nullptr;
-    b.n = 0;
-    c->held -= old;
+  drop(c, b);
+  cudaError_t e = scratch_alloc(c, b, bytes);
+  if (e == cudaErrorMemoryAllocation && !c->budget && &b != &c->wimg && &b != &c->stage && (c->wimg.p || c->stage.p)) {
+    cudaGetLastError();
+    drop_precompute(c);
+    e = scratch_alloc(c, b, bytes);
   }
-  cudaError_t e = cudaMalloc(&b.p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     b.p = nullptr;
@@ -163,27 +183,52 @@ int check_geometry_args(ecc_ctx* c, int n_views, const void* P, int W, int H, in
 }
 
 
-// Scratch of the many-view precompute: enough for ten groups of 32 views on a 620 x 480
-// detector, or for four on a 976 x 976 one.
+// Scratch of the many-view precompute in a context without a budget, FP16 staging included:
+// the weighted images of 13 groups of 32 views on the 768 x 768 grid of a 620 x 480 detector,
+// or of four on the 1024 x 1382 grid of a 976 x 976 one.
 constexpr size_t kViewsScratch = (size_t)1152 << 20;
 constexpr int kHostBatch = 128;  // views per upload of the host-buffer call
 
-// Scratch of a precompute and the plan that fits it: the many-view form on less and less
-// scratch, at last view by view, within the context's budget.
+// Chooses the plan of a precompute and allocates its scratch.  In a context with a budget no
+// buffer of the many-view form is larger than the view-by-view form's on the same call, so
+// that the budget holds whatever it held with that form, in every order of calls (buffers
+// only grow); less where the budget has less left.  Without a budget the form takes up to
+// kViewsScratch, and where the device has no such memory falls back to that.
 int ensure_precompute(ecc_ctx* c, int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
                       ecc::RadonPlan* plan) {
   int rc;
   if ((rc = ensure(c, c->views, sizeof(ecc::ViewRec) * (size_t)n_views, "views")) != ECC_OK) return rc;
-  size_t cap = kViewsScratch;
-  for (;;) {
-    *plan = ecc::radon_plan(n_views, W, H, n_alpha, n_s, dtype, max_batch, cap, 0);
-    plan->wait_ns = c->wait_ns;
-    rc = ensure(c, c->rtable, plan->table_bytes(n_views, n_alpha), "radon table");
-    if (rc == ECC_OK) rc = ensure(c, c->wimg, plan->wimg_bytes, "weighted images");
-    if (rc == ECC_OK && plan->stage_bytes) rc = ensure(c, c->stage, plan->stage_bytes, "FP16 staging");
-    if (rc == ECC_OK || !plan->views) return rc;
-    cap = plan->batch > 32 ? plan->wimg_bytes / 2 : plan->wimg_bytes - 1;
+  const ecc::RadonPlan by_view = ecc::radon_plan_by_view(n_views, W, H, n_alpha, n_s, dtype);
+  ecc::RadonRoom small;
+  small.wimg = by_view.wimg_bytes;
+  small.stage = by_view.stage_bytes;
+  if (c->budget) {
+    ecc::RadonPlan many{};
+    many.views = true;
+    const size_t left = c->budget - (c->held - c->rtable.n - c->wimg.n - c->stage.n);
+    const size_t table = std::max(c->rtable.n, many.table_bytes(n_views, n_alpha));
+    small.total = left > table ? left - table : 0;
   }
+  ecc::RadonRoom large;
+  large.total = kViewsScratch;
+  auto choose = [&](const ecc::RadonPlan& p) {
+    *plan = p;
+    plan->wait_ns = c->wait_ns;
+    rc = ensure(c, c->rtable, p.table_bytes(n_views, n_alpha), "radon table");
+    if (rc == ECC_OK) rc = ensure(c, c->wimg, p.wimg_bytes, "weighted images");
+    if (rc == ECC_OK && p.stage_bytes) rc = ensure(c, c->stage, p.stage_bytes, "FP16 staging");
+    return rc == ECC_OK;
+  };
+  if (!c->budget) {
+    const ecc::RadonPlan p = ecc::radon_plan(n_views, W, H, n_alpha, n_s, dtype, max_batch, large);
+    if (choose(p) || !p.views) return rc;
+    drop_precompute(c);
+  }
+  const ecc::RadonPlan p = ecc::radon_plan(n_views, W, H, n_alpha, n_s, dtype, max_batch, small);
+  if (choose(p) || !p.views) return rc;
+  if (!c->budget) drop_precompute(c);
+  choose(by_view);
+  return rc;
 }
 
 // batch_ready (or NULL): one event per batch of the plan, which the stream waits for
@@ -677,6 +722,17 @@ extern "C" int ecc_internal_set_wait_ns(ecc_ctx* c, unsigned long long ns) {
   c->wait_ns = ns;
   return ECC_OK;
 }
+
+// Internal (tests only): the context's scratch allocations fail as on a full device where
+// together they would exceed this many bytes (0: no such limit).
+extern "C" int ecc_internal_set_device_limit(ecc_ctx* c, size_t bytes) {
+  if (!c) return ECC_EINVAL;
+  c->device_limit = bytes;
+  return ECC_OK;
+}
+
+// Internal (tests only): bytes of scratch that the context holds.
+extern "C" size_t ecc_internal_held(const ecc_ctx* c) { return c ? c->held : 0; }
 
 extern "C" int ecc_internal_record_sizes(int* view_bytes, int* pair_bytes) {
   *view_bytes = (int)sizeof(ecc::ViewRec);

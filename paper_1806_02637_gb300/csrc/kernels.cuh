@@ -174,11 +174,16 @@ struct RadonPlan {
     return reinterpret_cast<RadonView*>(table + (size_t)copies(n_views) * n_alpha);
   }
 };
-// At most max_batch views per pass; wimg_cap bounds the many-view form's scratch and
-// total_cap (0: none) its scratch and staging together.  Where no group of views fits
-// the plan is the view-by-view form's.
-RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch, size_t wimg_cap,
-                     size_t total_cap);
+// Scratch that a many-view plan may take: weighted images, FP16 staging, and both together.
+struct RadonRoom {
+  size_t wimg = SIZE_MAX, stage = SIZE_MAX, total = SIZE_MAX;
+};
+// The many-view form in the largest groups that fit the room, at most max_batch views (in
+// groups of 32) per pass.  Where none fits, or the scan does not qualify, the plan is the
+// view-by-view form's, which follows neither limit.
+RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
+                     const RadonRoom& room);
+RadonPlan radon_plan_by_view(int n_views, int W, int H, int n_alpha, int n_s, int dtype);
 
 // Many-view form, in groups of 32 views.
 struct ViewsPlan {

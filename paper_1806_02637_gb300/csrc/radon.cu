@@ -331,32 +331,41 @@ size_t radon_f16_stage_bytes(int n_alpha, int n_s, int batch_views) {
   return sizeof(float) * (size_t)n_alpha * n_s * batch_views;
 }
 
-RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch, size_t wimg_cap,
-                     size_t total_cap) {
+static size_t stage_bytes(int n_alpha, int n_s, int dtype, int batch) {
+  return dtype == 1 ? radon_f16_stage_bytes(n_alpha, n_s, batch) : 0;
+}
+
+RadonPlan radon_plan_by_view(int n_views, int W, int H, int n_alpha, int n_s, int dtype) {
   RadonPlan p{};
-  auto stage = [&](int batch) { return dtype == 1 ? radon_f16_stage_bytes(n_alpha, n_s, batch) : (size_t)0; };
-  const int least = ViewsPlan::min_views(W, H, n_alpha, n_s);
-  if (least > 0 && n_views >= least) {
-    for (int axes = 2; axes >= 1; --axes) {
-      const size_t gb = ViewsPlan::group_bytes(axes, W, H, n_alpha, n_s);
-      int groups = (int)std::min<size_t>((size_t)(n_views + 31) / 32, wimg_cap / gb);
-      groups = std::min(groups, (max_batch + 31) / 32);
-      auto batch = [&] { return std::min(n_views, groups * 32); };
-      while (groups > 0 && total_cap && gb * groups + stage(batch()) > total_cap) --groups;
-      if (groups == 0) continue;
-      p.views = true;
-      p.batch = batch();
-      p.wimg_bytes = gb * groups;
-      p.stage_bytes = stage(p.batch);
-      return p;
-    }
-  }
   const size_t plane = radon_plane_bytes(W, H, n_s);
   const size_t max_batch_bytes = (size_t)256 << 20;  // weighted images of a batch, unless one view takes more
   p.batch = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_views, max_batch_bytes / plane));
   p.wimg_bytes = plane * (size_t)p.batch;
-  p.stage_bytes = stage(p.batch);
+  p.stage_bytes = stage_bytes(n_alpha, n_s, dtype, p.batch);
   return p;
+}
+
+RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
+                     const RadonRoom& room) {
+  const int least = ViewsPlan::min_views(W, H, n_alpha, n_s);
+  if (least > 0 && n_views >= least) {
+    for (int axes = 2; axes >= 1; --axes) {
+      const size_t gb = ViewsPlan::group_bytes(axes, W, H, n_alpha, n_s);
+      int groups = (int)std::min<size_t>((size_t)(n_views + 31) / 32, room.wimg / gb);
+      groups = std::min(groups, (max_batch + 31) / 32);
+      auto batch = [&] { return std::min(n_views, groups * 32); };
+      auto stage = [&] { return stage_bytes(n_alpha, n_s, dtype, batch()); };
+      while (groups > 0 && (stage() > room.stage || gb * groups + stage() > room.total)) --groups;
+      if (groups == 0) continue;
+      RadonPlan p{};
+      p.views = true;
+      p.batch = batch();
+      p.wimg_bytes = gb * groups;
+      p.stage_bytes = stage();
+      return p;
+    }
+  }
+  return radon_plan_by_view(n_views, W, H, n_alpha, n_s, dtype);
 }
 
 // FP16 storage of nb views staged in FP32: per-view maximum, scale, quantisation.

@@ -94,14 +94,15 @@ Layout layout_of(const ecc_job& j) {
   L.images = take(n * (size_t)j.W * j.H * sizeof(float));
   // The precompute's scratch is that of the view-by-view form, in which the many-view
   // form takes the largest groups that fit: a job's footprint does not depend on the form.
-  const ecc::RadonPlan by_view = ecc::radon_plan((int)n, j.W, j.H, j.n_alpha, j.n_s, j.dtype, (int)n, 0, 0);
+  const ecc::RadonPlan by_view = ecc::radon_plan_by_view((int)n, j.W, j.H, j.n_alpha, j.n_s, j.dtype);
   L.rtable = take(by_view.table_bytes((int)n, j.n_alpha));
   L.wimg = take(by_view.wimg_bytes);
   L.stage = take(by_view.stage_bytes);
   L.plan.views = true;
   const size_t wimg = align256(L.rtable + L.plan.table_bytes((int)n, j.n_alpha));
-  const size_t room = o - wimg - 256;
-  L.plan = ecc::radon_plan((int)n, j.W, j.H, j.n_alpha, j.n_s, j.dtype, (int)n, room, room);
+  ecc::RadonRoom room;
+  room.total = o - wimg - 256;
+  L.plan = ecc::radon_plan((int)n, j.W, j.H, j.n_alpha, j.n_s, j.dtype, (int)n, room);
   if (L.plan.views) {
     L.wimg = wimg;
     L.stage = wimg + align256(L.plan.wimg_bytes);
