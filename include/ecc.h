@@ -224,7 +224,8 @@ int ecc_evaluate_frozen(ecc_ctx* ctx, int n_views, const double* P, const double
  * the projections (host FP32 [n_views][H][W], pinned memory recommended) to the
  * device, computes the sinograms (ECC_F32, kept in the context) and the total
  * over all pairs a < b, and copies the total back into *total_host.  Synchronous:
- * returns after the result is on the host.
+ * returns after the result is on the host.  ECC_ETIMEOUT if a device wait of the
+ * precompute gave up (ecc_status() then has ECC_STATUS_TIMEOUT too).
  */
 int ecc_scan_consistency_host(ecc_ctx* ctx, int n_views, const double* P_host, const float* images_host, int W,
                               int H, int n_alpha, int n_s, int n_kappa, double cauchy_c, double* total_host,

@@ -42,7 +42,14 @@ struct ecc_ctx {
   unsigned long long wait_ns = ecc::kWaitNs;  // limit of the precompute's device waits
   size_t device_limit = 0;                    // tests: allocations beyond it fail as on a full device
   std::string err;
-  int* d_status = nullptr;
+  // status words and the total of the host-buffer call
+  struct Report {
+    int status;  // accumulated until ecc_status reads it
+    int call;    // of a host-buffer call alone, joined into status at its end
+    double total;
+  };
+  Report* report = nullptr;  // device
+  int* d_status = nullptr;   // the word that launches set: report->status, or report->call
   Buf views, pairs, ctile, adir, perpair, nk, partial, rtable, wimg, stage;
   Buf vtan, Gpp, gq;  // adjoint scratch: view tangents (theta), d e / d A, d e / d (C, up, cofc)
   Buf vtanP;          // view tangents with respect to P
@@ -54,7 +61,7 @@ struct ecc_ctx {
   bool samp_valid = false;
   int samp_views = 0, samp_pairs = 0, samp_K = 0, samp_W = 0, samp_H = 0;
   const void* samp_pair_ptr = nullptr;
-  Buf h_P, h_img, h_sino, h_total;  // buffers of the host-buffer entry point
+  Buf h_P, h_img, h_sino;  // buffers of the host-buffer entry point
   cudaStream_t copy_stream = nullptr;  // its image uploads, per precompute batch
   ecc_serve* serve = nullptr;       // serving scheduler, created by the first ecc_submit
 };
@@ -392,13 +399,14 @@ int ecc_create(ecc_ctx** out, int device, size_t hbm_budget_bytes) {
   ecc_ctx* c = new ecc_ctx();
   c->device = device;
   c->budget = hbm_budget_bytes;
-  e = cudaMalloc(&c->d_status, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int));
+  e = cudaMalloc(&c->report, sizeof(ecc_ctx::Report));
+  if (e == cudaSuccess) e = cudaMemset(c->report, 0, sizeof(ecc_ctx::Report));
   if (e != cudaSuccess) {
     cudaGetLastError();
     delete c;
     return fail(nullptr, ECC_ECUDA, "context allocation: %s", cudaGetErrorString(e));
   }
+  c->d_status = &c->report->status;
   *out = c;
   return ECC_OK;
 }
@@ -409,10 +417,10 @@ void ecc_destroy(ecc_ctx* c) {
   ecc::serve_destroy(c->serve);
   cudaDeviceSynchronize();
   Buf* bufs[] = {&c->views, &c->pairs, &c->ctile, &c->adir, &c->perpair, &c->nk, &c->partial, &c->rtable, &c->wimg,
-                 &c->vtan, &c->Gpp, &c->gq, &c->vtanP, &c->stage, &c->h_P, &c->h_img, &c->h_sino, &c->h_total};
+                 &c->vtan, &c->Gpp, &c->gq, &c->vtanP, &c->stage, &c->h_P, &c->h_img, &c->h_sino};
   for (Buf* b : bufs)
     if (b->p) cudaFree(b->p);
-  if (c->d_status) cudaFree(c->d_status);
+  if (c->report) cudaFree(c->report);
   for (const ProfRec& r : c->recs) {
     if (r.b) cudaEventDestroy(r.b);
     if (r.e) cudaEventDestroy(r.e);
@@ -588,8 +596,15 @@ int ecc_scan_consistency_host(ecc_ctx* c, int n_views, const double* P_host, con
   if ((rc = ensure(c, c->h_P, pb, "host-call P")) != ECC_OK) return rc;
   if ((rc = ensure(c, c->h_img, ib, "host-call images")) != ECC_OK) return rc;
   if ((rc = ensure(c, c->h_sino, sb, "host-call sinograms")) != ECC_OK) return rc;
-  if ((rc = ensure(c, c->h_total, sizeof(double), "host-call total")) != ECC_OK) return rc;
-  cudaError_t e = cudaMemcpyAsync(c->h_P.p, P_host, pb, cudaMemcpyHostToDevice, s);
+  // the call's own status bits, so that it reports a wait that gave up, not an earlier call's
+  struct OwnStatus {
+    ecc_ctx* c;
+    ~OwnStatus() { c->d_status = &c->report->status; }
+  } own{c};
+  c->d_status = &c->report->call;
+  cudaError_t e = cudaMemsetAsync(c->d_status, 0, sizeof(int), s);
+  if (e != cudaSuccess) return cuda_fail(c, e, "status reset");
+  e = cudaMemcpyAsync(c->h_P.p, P_host, pb, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "host-to-device copy");
   // From pinned host memory the images go up per precompute batch on a second stream,
   // so that the upload of batch b + 1 overlaps the projection of batch b; pageable
@@ -634,12 +649,19 @@ int ecc_scan_consistency_host(ecc_ctx* c, int n_views, const double* P_host, con
                       c->h_sino.p, nullptr, plan, s, ready.ev.empty() ? nullptr : ready.ev.data());
   if (rc != ECC_OK) return rc;
   rc = run_evaluate(c, n_views, (const double*)c->h_P.p, nullptr, c->h_sino.p, nullptr, W, H, n_alpha, n_s, ECC_F32,
-                    n_kappa, cauchy_c, nullptr, (int)np, (double*)c->h_total.p, nullptr, nullptr, nullptr, nullptr, false,
-                    s);
+                    n_kappa, cauchy_c, nullptr, (int)np, &c->report->total, nullptr, nullptr, nullptr, nullptr, false, s);
   if (rc != ECC_OK) return rc;
-  e = cudaMemcpyAsync(total_host, c->h_total.p, sizeof(double), cudaMemcpyDeviceToHost, s);
+  ecc_ctx::Report r;
+  e = cudaMemcpyAsync(&r, c->report, sizeof r, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess && r.call) {
+    r.status |= r.call;
+    e = cudaMemcpyAsync(&c->report->status, &r.status, sizeof(int), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  }
   if (e != cudaSuccess) return cuda_fail(c, e, "device-to-host copy");
+  if (r.call & ecc::kStatusTimeout) return fail(c, ECC_ETIMEOUT, "a device wait of the precompute gave up");
+  *total_host = r.total;
   return ECC_OK;
 }
 

@@ -39,3 +39,22 @@ def test_a_wait_that_gives_up_is_reported_and_the_next_call_is_whole(n, W, Hh, n
             again, _ = ecc.ecc_precompute_radon_derivative(ctx, P, images, n_alpha, n_s)
             assert ecc.ecc_status(ctx) == 0
             assert torch.equal(again, S)
+
+
+def test_the_call_from_host_buffers_reports_its_own_wait():
+    """ecc_scan_consistency_host is synchronous: a wait that gave up in it is its error, and a bit left by an
+    earlier call is not."""
+    import paper_1806_02637_gb300 as ecc
+    P, images = views._scan(40, 300, 260, 18)
+    with ecc.Context(0) as ctx:
+        total = ecc.ecc_scan_consistency_host(ctx, P, images, 512, 400, 65)
+        _set_wait_ns(ctx, 0)
+        with pytest.raises(ecc.EccError, match=r"\(-4\)"):
+            ecc.ecc_scan_consistency_host(ctx, P, images, 512, 400, 65)
+        _set_wait_ns(ctx, 10 ** 9)
+        assert ecc.ecc_scan_consistency_host(ctx, P, images, 512, 400, 65) == total
+        assert ecc.ecc_status(ctx) & TIMEOUT
+        assert ecc.ecc_status(ctx) == 0
+        P[0] = float("nan")   # other bits go on to ecc_status as before
+        ecc.ecc_scan_consistency_host(ctx, P, images, 512, 400, 65)
+        assert ecc.ecc_status(ctx) & 1
