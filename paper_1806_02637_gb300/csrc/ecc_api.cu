@@ -194,7 +194,12 @@ int check_geometry_args(ecc_ctx* c, int n_views, const void* P, int W, int H, in
 // the weighted images of 13 groups of 32 views on the 768 x 768 grid of a 620 x 480 detector,
 // or of four on the 1024 x 1382 grid of a 976 x 976 one.
 constexpr size_t kViewsScratch = (size_t)1152 << 20;
-constexpr int kHostBatch = 128;  // views per upload of the host-buffer call
+// Views per upload of the host-buffer call, and of its first, which nothing overlaps.  The line
+// sums of one group (1.85 ms on 620 x 480) take longer than the upload of the next 256 views
+// (1.5 ms at 205 GB/s), and each pass costs about 0.4 ms in weights and a last wave: 496 views
+// in passes of 32 and 256 take 24.75 ms, of 32 and 128 25.6, of 128 25.7, of 464 25.3, without
+// uploads 24.15.
+constexpr int kHostBatch = 256, kHostLead = 32;
 
 // Chooses the plan of a precompute and allocates its scratch.  In a context with a budget no
 // buffer of the many-view form is larger than the view-by-view form's on the same call, so
@@ -238,8 +243,8 @@ int ensure_precompute(ecc_ctx* c, int n_views, int W, int H, int n_alpha, int n_
   return rc;
 }
 
-// batch_ready (or NULL): one event per batch of the plan, which the stream waits for
-// before the batch reads its images.
+// batch_ready (or NULL): one event per pass of the plan, which the stream waits for
+// before the pass reads its images.
 int run_precompute(ecc_ctx* c, int n_views, const double* P, const float* images, int W, int H, int n_alpha, int n_s,
                    int dtype, void* sino_out, float* scales_out, const ecc::RadonPlan& plan, cudaStream_t s,
                    const cudaEvent_t* batch_ready = nullptr) {
@@ -611,8 +616,8 @@ int ecc_scan_consistency_host(ecc_ctx* c, int n_views, const double* P_host, con
   // memory (whose asynchronous copies block the host) is copied in one piece.
   ecc::RadonPlan plan;
   if ((rc = ensure_precompute(c, n_views, W, H, n_alpha, n_s, ECC_F32, kHostBatch, &plan)) != ECC_OK) return rc;
-  const int batch = plan.batch;
-  const int n_batches = (n_views + batch - 1) / batch;
+  if (plan.views) plan.lead = std::min(plan.batch, kHostLead);
+  const int n_batches = plan.passes(n_views);
   cudaPointerAttributes pa;
   const bool pinned = cudaPointerGetAttributes(&pa, images_host) == cudaSuccess && pa.type == cudaMemoryTypeHost;
   (void)cudaGetLastError();  // a pageable pointer may leave an error from the query
@@ -635,7 +640,7 @@ int ecc_scan_consistency_host(ecc_ctx* c, int n_views, const double* P_host, con
     e = cudaEventRecord(ready.ev[n_batches], s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->copy_stream, ready.ev[n_batches], 0);
     for (int b = 0; b < n_batches && e == cudaSuccess; ++b) {
-      const size_t v0 = (size_t)b * batch, nv = (size_t)std::min(batch, n_views - b * batch);
+      const size_t v0 = (size_t)plan.begin(b), nv = (size_t)plan.count(b, n_views);
       const size_t px = (size_t)W * H;
       e = cudaMemcpyAsync((float*)c->h_img.p + v0 * px, images_host + v0 * px, sizeof(float) * px * nv,
                           cudaMemcpyHostToDevice, c->copy_stream);

@@ -1,5 +1,6 @@
 // Kernel declarations shared by the translation units of the library.
 #pragma once
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cuda_bf16.h>
@@ -163,6 +164,10 @@ struct RadonPlan {
   unsigned long long wait_ns = kWaitNs;
   bool views;          // many views at once
   int batch;           // views per pass over the scratch
+  int lead;            // views of the first pass
+  int passes(int n_views) const { return n_views <= lead ? 1 : 1 + (n_views - lead + batch - 1) / batch; }
+  int begin(int pass) const { return pass == 0 ? 0 : lead + (pass - 1) * batch; }
+  int count(int pass, int n_views) const { return std::min(pass == 0 ? lead : batch, n_views - begin(pass)); }
   size_t wimg_bytes;   // weighted images
   size_t stage_bytes;  // FP32 staging of FP16 storage
   // the line table (copies of n_alpha rows) and the per-view weights after it
@@ -201,7 +206,7 @@ cudaError_t launch_pair_setup(int n_views, long long n_pairs, const int32_t* pai
 cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_alpha, int n_s, int dtype,
                          void* sino_out, float* scales_out, const RadonRow* table, void* wimg, float* stage,
                          const RadonPlan& plan, int* status, const LaunchHooks& hooks, cudaStream_t stream,
-                         const cudaEvent_t* batch_ready = nullptr);  // per batch: wait before reading its images
+                         const cudaEvent_t* batch_ready = nullptr);  // per pass: wait before reading its images
 cudaError_t launch_radon_views(const RadonRow* table, const RadonView* rv, int n_views, const float* images, int W,
                                int H, int n_alpha, int n_s, void* planes, size_t plane_bytes, float* of,
                                __nv_bfloat16* ob, int* status, unsigned long long wait_ns, bool behind,

@@ -340,6 +340,7 @@ RadonPlan radon_plan_by_view(int n_views, int W, int H, int n_alpha, int n_s, in
   const size_t plane = radon_plane_bytes(W, H, n_s);
   const size_t max_batch_bytes = (size_t)256 << 20;  // weighted images of a batch, unless one view takes more
   p.batch = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_views, max_batch_bytes / plane));
+  p.lead = p.batch;
   p.wimg_bytes = plane * (size_t)p.batch;
   p.stage_bytes = stage_bytes(n_alpha, n_s, dtype, p.batch);
   return p;
@@ -359,7 +360,7 @@ RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype,
       if (groups == 0) continue;
       RadonPlan p{};
       p.views = true;
-      p.batch = batch();
+      p.batch = p.lead = batch();
       p.wimg_bytes = gb * groups;
       p.stage_bytes = stage();
       return p;
@@ -406,10 +407,10 @@ cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_a
   const size_t per_view = (size_t)n_alpha * n_s;
   float2* wv = reinterpret_cast<float2*>(wimg);
   const bool behind = batch_ready == nullptr;  // behind an event a batch's first kernel is launched plainly
-  for (int v0 = 0; v0 < n_views; v0 += plan.batch) {
-    const int nb = min(plan.batch, n_views - v0);
+  for (int pass = 0; pass < plan.passes(n_views); ++pass) {
+    const int v0 = plan.begin(pass), nb = plan.count(pass, n_views);
     cudaError_t e;
-    if (batch_ready && (e = cudaStreamWaitEvent(stream, batch_ready[v0 / plan.batch], 0)) != cudaSuccess) return e;
+    if (batch_ready && (e = cudaStreamWaitEvent(stream, batch_ready[pass], 0)) != cudaSuccess) return e;
     const float* im = images + (size_t)v0 * W * H;
     const size_t oo = (size_t)v0 * per_view;
     float* of = dtype == 0 ? (float*)sino_out + oo : (dtype == 1 ? stage : nullptr);

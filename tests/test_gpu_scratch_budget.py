@@ -121,3 +121,19 @@ def test_many_small_and_many_large_calls_in_one_budget(scan):
                 for dtype in order:
                     ecc.ecc_precompute_radon_derivative(ctx, P[:n], images[:n], N_ALPHA, N_S, dtype=dtype)
             assert ecc.ecc_status(ctx) == 0
+
+
+def test_fp16_short_scan_in_every_budget_from_the_least():
+    """The 496-view short scan in FP16: line sums and staging of one group take more than 256 MiB here."""
+    import paper_1806_02637_gb300 as ecc
+    import synth
+    c = synth.CONFIGS["c2"]
+    images = torch.randn((c.n_views, c.H, c.W), device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    P = torch.from_numpy(synth.trajectory(c)).cuda()
+    out = torch.empty((c.n_views, c.n_alpha, c.n_s), dtype=torch.float16, device="cuda")
+    with ecc.Context(0) as ctx:
+        want, scales = ecc.ecc_precompute_radon_derivative(ctx, P, images, c.n_alpha, c.n_s, dtype=out.dtype)
+    for room in range(390 * MIB, 1200 * MIB, 35 * MIB):   # 376 MiB view by view
+        with ecc.Context(0, hbm_budget_bytes=room) as ctx:
+            S, s = ecc.ecc_precompute_radon_derivative(ctx, P, images, c.n_alpha, c.n_s, dtype=out.dtype, out=out)
+            assert torch.equal(S, want) and torch.equal(s, scales), room
