@@ -126,10 +126,26 @@ int ecc_profile_read(ecc_ctx* ctx, void* stream, int max_entries, char* names, l
  *            value = S / scale rounded to FP16; required for ECC_F16, ignored
  *            otherwise.  F32 and BF16 store S itself (BF16 rounded to nearest).
  * Limits: 2 <= W, H <= 16384; 4 <= n_alpha <= 65535; 2 <= n_s <= 65535.
+ *
+ * S of a view depends on that view alone, but it is summed in one of two forms, whose
+ * roundings differ (by 1e-6 of max |S| or so): calls with enough views on a grid that
+ * allows it follow each detector line once for 32 views, others go view by view.  A
+ * context whose memory budget has no room for 32 views at once goes view by view too,
+ * as does a served job whose scratch (that of the view-by-view form) has none.
  */
 int ecc_precompute_radon_derivative(ecc_ctx* ctx, int n_views, const double* P, const float* images, int W, int H,
                                     int n_alpha, int n_s, int dtype, void* sino_out, float* scales_out,
                                     void* stream);
+
+/*
+ * As ecc_precompute_radon_derivative, for n_views of the views of a scan that has
+ * n_scan_views (>= n_views) in all: the form is the whole scan's, so that in contexts
+ * without a budget the sinograms are bit for bit those of one call on all views, however
+ * the scan is divided over calls or ranks.
+ */
+int ecc_precompute_radon_derivative_part(ecc_ctx* ctx, int n_scan_views, int n_views, const double* P,
+                                         const float* images, int W, int H, int n_alpha, int n_s, int dtype,
+                                         void* sino_out, float* scales_out, void* stream);
 
 /*
  * Epipolar consistency over a list of view pairs (Eq. 15-17).

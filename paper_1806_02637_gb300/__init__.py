@@ -84,6 +84,8 @@ def load(build_if_missing: bool = True):
         lib.ecc_status.restype = i
         lib.ecc_precompute_radon_derivative.argtypes = [vp, i, vp, vp, i, i, i, i, i, vp, vp, vp]
         lib.ecc_precompute_radon_derivative.restype = i
+        lib.ecc_precompute_radon_derivative_part.argtypes = [vp, i, i, vp, vp, i, i, i, i, i, vp, vp, vp]
+        lib.ecc_precompute_radon_derivative_part.restype = i
         lib.ecc_evaluate.argtypes = [vp, i, vp, vp, vp, vp, i, i, i, i, i, i, d, vp, i, vp, vp, vp, vp]
         lib.ecc_evaluate.restype = i
         lib.ecc_scan_consistency_host.argtypes = [vp, i, vp, vp, i, i, i, i, i, d, ctypes.POINTER(d), vp]
@@ -212,9 +214,11 @@ class Context:
 
 
 def ecc_precompute_radon_derivative(ctx: Context, P, images, n_alpha: int, n_s: int, dtype=None, out=None,
-                                    scales=None, stream=None):
+                                    scales=None, stream=None, scan_views=None):
     """S_lambda on the (alpha, s) grid for every view.  P: CUDA float64 [N,3,4];
-    images: CUDA float32 [N,H,W].  Returns (sino [N,n_alpha,n_s], scales or None)."""
+    images: CUDA float32 [N,H,W].  Returns (sino [N,n_alpha,n_s], scales or None).
+    scan_views: where these are some views of a larger scan, the number of all its views:
+    without a memory budget the result is then, bit for bit, that of one call on all of them."""
     torch = _torch()
     dtype = dtype or torch.float32
     code = _dtype_code(dtype)
@@ -230,8 +234,9 @@ def ecc_precompute_radon_derivative(ctx: Context, P, images, n_alpha: int, n_s: 
         _dev(scales, torch.float32, "scales", (N,))
     else:
         scales = None
-    rc = load().ecc_precompute_radon_derivative(ctx.handle, N, _ptr(P), _ptr(images), W, H, int(n_alpha), int(n_s),
-                                                code, _ptr(out), _ptr(scales), _stream(stream))
+    rc = load().ecc_precompute_radon_derivative_part(ctx.handle, N if scan_views is None else int(scan_views), N,
+                                                     _ptr(P), _ptr(images), W, H, int(n_alpha), int(n_s), code,
+                                                     _ptr(out), _ptr(scales), _stream(stream))
     _check(ctx, rc, "ecc_precompute_radon_derivative")
     return out, scales
 

@@ -205,8 +205,9 @@ constexpr int kHostBatch = 256, kHostLead = 32;
 // buffer of the many-view form is larger than the view-by-view form's on the same call, so
 // that the budget holds whatever it held with that form, in every order of calls (buffers
 // only grow); less where the budget has less left.  Without a budget the form takes up to
-// kViewsScratch, and where the device has no such memory falls back to that.
-int ensure_precompute(ecc_ctx* c, int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
+// kViewsScratch, and where the device has no such memory falls back to that.  n_scan: views of
+// the scan that these are part of.
+int ensure_precompute(ecc_ctx* c, int n_scan, int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
                       ecc::RadonPlan* plan) {
   int rc;
   if ((rc = ensure(c, c->views, sizeof(ecc::ViewRec) * (size_t)n_views, "views")) != ECC_OK) return rc;
@@ -232,11 +233,11 @@ int ensure_precompute(ecc_ctx* c, int n_views, int W, int H, int n_alpha, int n_
     return rc == ECC_OK;
   };
   if (!c->budget) {
-    const ecc::RadonPlan p = ecc::radon_plan(n_views, W, H, n_alpha, n_s, dtype, max_batch, large);
+    const ecc::RadonPlan p = ecc::radon_plan(n_scan, n_views, W, H, n_alpha, n_s, dtype, max_batch, large);
     if (choose(p) || !p.views) return rc;
     drop_precompute(c);
   }
-  const ecc::RadonPlan p = ecc::radon_plan(n_views, W, H, n_alpha, n_s, dtype, max_batch, small);
+  const ecc::RadonPlan p = ecc::radon_plan(n_scan, n_views, W, H, n_alpha, n_s, dtype, max_batch, small);
   if (choose(p) || !p.views) return rc;
   if (!c->budget) drop_precompute(c);
   choose(by_view);
@@ -500,14 +501,23 @@ int ecc_profile_read(ecc_ctx* c, void* stream, int max_entries, char* names, lon
 int ecc_precompute_radon_derivative(ecc_ctx* c, int n_views, const double* P, const float* images, int W, int H,
                                     int n_alpha, int n_s, int dtype, void* sino_out, float* scales_out,
                                     void* stream) {
+  return ecc_precompute_radon_derivative_part(c, n_views, n_views, P, images, W, H, n_alpha, n_s, dtype, sino_out,
+                                              scales_out, stream);
+}
+
+int ecc_precompute_radon_derivative_part(ecc_ctx* c, int n_scan_views, int n_views, const double* P,
+                                         const float* images, int W, int H, int n_alpha, int n_s, int dtype,
+                                         void* sino_out, float* scales_out, void* stream) {
   if (!c) return fail(nullptr, ECC_EINVAL, "ctx is NULL");
   int rc = check_geometry_args(c, n_views, P, W, H, n_alpha, n_s, dtype);
   if (rc != ECC_OK) return rc;
+  if (n_scan_views < n_views) return fail(c, ECC_EINVAL, "n_scan_views %d < n_views %d", n_scan_views, n_views);
   if (!images || !sino_out) return fail(c, ECC_EINVAL, "images or sino_out is NULL");
   if (dtype == ECC_F16 && !scales_out) return fail(c, ECC_EINVAL, "ECC_F16 needs scales_out");
   DeviceGuard g(c->device);
   ecc::RadonPlan plan;
-  if ((rc = ensure_precompute(c, n_views, W, H, n_alpha, n_s, dtype, n_views, &plan)) != ECC_OK) return rc;
+  if ((rc = ensure_precompute(c, n_scan_views, n_views, W, H, n_alpha, n_s, dtype, n_views, &plan)) != ECC_OK)
+    return rc;
   return run_precompute(c, n_views, P, images, W, H, n_alpha, n_s, dtype, sino_out, scales_out, plan,
                         (cudaStream_t)stream);
 }
@@ -615,7 +625,7 @@ int ecc_scan_consistency_host(ecc_ctx* c, int n_views, const double* P_host, con
   // so that the upload of batch b + 1 overlaps the projection of batch b; pageable
   // memory (whose asynchronous copies block the host) is copied in one piece.
   ecc::RadonPlan plan;
-  if ((rc = ensure_precompute(c, n_views, W, H, n_alpha, n_s, ECC_F32, kHostBatch, &plan)) != ECC_OK) return rc;
+  if ((rc = ensure_precompute(c, n_views, n_views, W, H, n_alpha, n_s, ECC_F32, kHostBatch, &plan)) != ECC_OK) return rc;
   if (plan.views) plan.lead = std::min(plan.batch, kHostLead);
   const int n_batches = plan.passes(n_views);
   cudaPointerAttributes pa;

@@ -154,11 +154,11 @@ inline void pair_args_grid(PairArgs& g, int n_alpha, int n_s, int W, int H) {
   g.half_lo = (float)(half - (double)g.half_hi);
 }
 
-// How a dRadon/ds precompute runs, by its sizes and the scratch it may use.  Scans with
-// enough views whose grid qualifies follow the detector lines once for many views
-// (radon_views.cu), others view by view (radon.cu).  The choice between the two
-// depends on the sizes alone, and the many-view sums do not depend on how the views are
-// grouped, so that a scan's sinograms are the same wherever they are computed.
+// How a dRadon/ds precompute runs.  Scans with enough views whose grid qualifies follow the
+// detector lines once for many views (radon_views.cu), others view by view (radon.cu); the
+// two round differently.  The choice depends on the grid, on the number of views of the scan
+// (n_scan: of this call, or of the scan that the call's views are part of) and on the scratch
+// that the call may take.  The many-view sums do not depend on how the views are grouped.
 constexpr unsigned long long kWaitNs = 1000000000ull;  // a bounded device wait gives up after this long
 struct RadonPlan {
   unsigned long long wait_ns = kWaitNs;
@@ -186,7 +186,7 @@ struct RadonRoom {
 // The many-view form in the largest groups that fit the room, at most max_batch views (in
 // groups of 32) per pass.  Where none fits, or the scan does not qualify, the plan is the
 // view-by-view form's, which follows neither limit.
-RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
+RadonPlan radon_plan(int n_scan, int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
                      const RadonRoom& room);
 RadonPlan radon_plan_by_view(int n_views, int W, int H, int n_alpha, int n_s, int dtype);
 

@@ -346,10 +346,10 @@ RadonPlan radon_plan_by_view(int n_views, int W, int H, int n_alpha, int n_s, in
   return p;
 }
 
-RadonPlan radon_plan(int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
+RadonPlan radon_plan(int n_scan, int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
                      const RadonRoom& room) {
   const int least = ViewsPlan::min_views(W, H, n_alpha, n_s);
-  if (least > 0 && n_views >= least) {
+  if (least > 0 && n_scan >= least) {
     for (int axes = 2; axes >= 1; --axes) {
       const size_t gb = ViewsPlan::group_bytes(axes, W, H, n_alpha, n_s);
       int groups = (int)std::min<size_t>((size_t)(n_views + 31) / 32, room.wimg / gb);

@@ -4,7 +4,8 @@ Eq. 17 sums independent pair terms, and each view's S (Eq. 1) depends on that vi
 alone, so the path splits in two exchange steps:
 
 1. the views are split into contiguous slices, one per rank; each rank computes the
-   dRadon/ds sinograms of its slice, and an all-gather gives every rank all of them
+   dRadon/ds sinograms of its slice (in the form that the whole scan takes, so that they
+   are those of one GPU bit for bit), and an all-gather gives every rank all of them
    (on one GB300 the 496-view scan's FP32 sinograms are 1.17 GB, the 1240-view
    scan's FP16 ones 2.8 GB: every rank can hold all of them);
 2. the upper-triangular pair matrix is cut into view-block x view-block tiles and
@@ -123,7 +124,8 @@ def sharded_consistency(ctx, P, images, W: int, H: int, n_alpha: int, n_s: int, 
         raise ValueError("sharded_consistency takes FP32 or BF16 storage")
     n = P.shape[0]
     b, e = view_slices(n, world)[rank]
-    local, _ = ecc_precompute_radon_derivative(ctx, P[b:e], images[b:e], n_alpha, n_s, dtype=dtype)
+    local, _ = ecc_precompute_radon_derivative(ctx, P[b:e], images[b:e], n_alpha, n_s, dtype=dtype,
+                                                scan_views=n)
     sino = all_gather_views(local, n, world, group)
     pairs = torch.from_numpy(rank_pairs(n, world, rank, blocks_per_rank)).to(P.device)
     if with_grad:
