@@ -1138,8 +1138,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, GRAD ? 2 : 4) ecc_pair_ke
 }
 
 // The total of a call without gradients.
-__global__ void __launch_bounds__(1024) reduce_kernel(const double* __restrict__ partial, int n,
-                                                      double* __restrict__ total) {
+__global__ void __launch_bounds__(1024) reduce_kernel(const double* partial, int n, double* __restrict__ total) {
   wait_for_previous();
   __shared__ double s[kSumSlots];
   reduce_fixed<1024>(partial, n, total, s);

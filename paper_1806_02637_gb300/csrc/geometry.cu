@@ -773,7 +773,7 @@ cudaError_t launch_pair_setup(int n_views, long long n_pairs, const int32_t* pai
 // G = d e / d A (the pair kernel's adjoint, FP32 values): A = cofc [w v] is linear in
 // cofc, and the frame (w, v) is differentiated in reverse mode
 // (pencil_frame_adjoint_df).  Double-float throughout; out holds (hi, lo) pairs.
-__device__ void pair_grad_q(const PairRec& pr, const ViewRec* __restrict__ views, const double* __restrict__ G,
+__device__ void pair_grad_q(const PairRec& pr, const ViewRec* views, const double* G,
                             float2* __restrict__ out) {
   if (pr.status != 0 || pr.nk <= 0) {
     for (int j = 0; j < 30; ++j) out[j] = make_float2(0.0f, 0.0f);
@@ -817,8 +817,8 @@ __device__ void pair_grad_q(const PairRec& pr, const ViewRec* __restrict__ views
 // The first block sums the total meanwhile (a launch of its own before this one held up the
 // gradient by 8 us).
 __global__ void __launch_bounds__(kGradQThreads)
-    pair_grad_q_kernel(long long n_pairs, const PairRec* __restrict__ prs, const ViewRec* __restrict__ views,
-                       const double* __restrict__ Gpp, float2* __restrict__ gq, const double* __restrict__ partial,
+    pair_grad_q_kernel(long long n_pairs, const PairRec* prs, const ViewRec* views, const double* Gpp,
+                       float2* __restrict__ gq, const double* partial,
                        int n_partial, double* __restrict__ total) {
   __shared__ double s[kSumSlots];
   wait_for_previous();
@@ -836,7 +836,7 @@ __global__ void __launch_bounds__(kGradQThreads)
 // lam as a (hi, lo) pair.  With pairs == NULL the pairs of a view are found by the
 // row-major a < b enumeration, otherwise by scanning the pair list.
 __device__ void reduce_q_block(int lam, int n_views, long long n_pairs, const int32_t* __restrict__ pairs,
-                               const float2* __restrict__ gq, float2 (*sh)[256]) {
+                               const float2* gq, float2 (*sh)[256]) {
   df acc[15];
   for (int k = 0; k < 15; ++k) acc[k] = df{0.0f, 0.0f};
   auto add = [&](const float2* q) {
@@ -893,8 +893,7 @@ __device__ __forceinline__ double contract_theta(const float2 (*sh)[256], const 
 // grad[view][6] = d total / d theta (one block of 256 threads per view).
 __global__ void __launch_bounds__(256) view_grad_theta_kernel(int n_views, long long n_pairs,
                                                               const int32_t* __restrict__ pairs,
-                                                              const float2* __restrict__ gq,
-                                                              const ViewTan* __restrict__ vtan,
+                                                              const float2* gq, const ViewTan* vtan,
                                                               double* __restrict__ grad) {
   wait_for_previous();
   __shared__ float2 sh[15][256];
@@ -906,8 +905,7 @@ __global__ void __launch_bounds__(256) view_grad_theta_kernel(int n_views, long 
 // grad_P[view][12] = d total / d P (one block of 256 threads per view).
 __global__ void __launch_bounds__(256) view_grad_P_kernel(int n_views, long long n_pairs,
                                                           const int32_t* __restrict__ pairs,
-                                                          const float2* __restrict__ gq,
-                                                          const ViewTanP* __restrict__ vtan,
+                                                          const float2* gq, const ViewTanP* vtan,
                                                           double* __restrict__ grad_P) {
   wait_for_previous();
   __shared__ float2 sh[15][256];

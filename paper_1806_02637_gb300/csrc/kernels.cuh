@@ -66,10 +66,12 @@ struct LaunchHooks {
 
 // Kernels of a call that are launched behind the one before (programmatic dependent launch)
 // wait for its end and its stores as their first step: their launch and their blocks' start
-// overlap its end.  That takes 2 us to 5 us off a call of several short kernels (motion
-// gradient of 248 views 285 -> 282 us, evaluation of one pair 37.2 -> 35.0 us, two-view
-// precompute 43.8 -> 40.8 us).  Launched plainly: the first kernel of a call, which waits for
-// whatever the stream did before; pair_setup_kernel and ecc_pair_kernel, because an SM that
+// overlap its end.  What earlier kernels write is then not read-only for their duration: they
+// take it through pointers without const __restrict__ and never through __ldg, whose loads may
+// be non-coherent and may move ahead of the wait.  Starting early takes 2 us to 5 us off a
+// call of several short kernels (motion gradient of 248 views 285 -> 282 us, evaluation of one
+// pair 37.2 -> 35.0 us, two-view precompute 43.8 -> 40.8 us).  Launched plainly: the first
+// kernel of a call, which waits for whatever the stream did before; pair_setup_kernel and ecc_pair_kernel, because an SM that
 // never falls idle between them keeps the first one's split of L1 and shared memory, at which
 // fewer blocks of the second fit (evaluation of the 496-view scan 567 -> 747 us).
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -101,7 +103,7 @@ void launch_behind(void (*kernel)(K...), dim3 grid, dim3 block, size_t shared, c
 // slots, one after the other, then a tree, whatever THREADS.
 constexpr int kSumSlots = 1024;
 template <int THREADS>
-__device__ __forceinline__ void reduce_fixed(const double* __restrict__ partial, int n, double* __restrict__ total,
+__device__ __forceinline__ void reduce_fixed(const double* partial, int n, double* __restrict__ total,
                                              double* s) {
   const int per = (n + kSumSlots - 1) / kSumSlots;
 #pragma unroll 4

@@ -38,7 +38,7 @@ namespace {
 // pairs starting one pixel before the image; the weighted values of a 33x33 tile
 // are computed once into shared memory and both planes are written coalesced.  The
 // blocks beside the margins write their zeros.
-__global__ void weight_kernel(const float* __restrict__ images, const RadonView* __restrict__ rv, int W, int H,
+__global__ void weight_kernel(const float* __restrict__ images, const RadonView* rv, int W, int H,
                               int pad, int pitch_r, int pitch_c, float2* __restrict__ wimg, size_t plane) {
   wait_for_previous();
   __shared__ float tile[33][34];
@@ -127,7 +127,7 @@ struct JosephArgs {
 
 // Taps of rows u in [ua, ub) of one anchor block (all 16 rows when FULL).
 template <bool CLAMP, bool FULL>
-__device__ __forceinline__ void joseph_block(const float2* __restrict__ rp, float f0, float dyf, float lo_c, float hi_c,
+__device__ __forceinline__ void joseph_block(const float2* rp, float f0, float dyf, float lo_c, float hi_c,
                                              const float (&Mu)[kRowsPerAnchor], int ua, int ub, float& acc,
                                              float& comp) {
 #pragma unroll
@@ -141,7 +141,7 @@ __device__ __forceinline__ void joseph_block(const float2* __restrict__ rp, floa
         if (CLAMP) xf = fminf(fmaxf(xf, lo_c), hi_c);
         const float t = __fadd_rd(xf, Mu[u]);
         const float f = xf - (t - Mu[u]);
-        const float2 vd = __ldg(rp + __float_as_uint(t));
+        const float2 vd = rp[__float_as_uint(t)];
         s += fmaf(f, vd.y, vd.x);
       }
     }
@@ -157,9 +157,9 @@ __device__ __forceinline__ void joseph_block(const float2* __restrict__ rp, floa
 // slower on two.  (Several warps along one line, and the next rows' loads issued before these
 // rows' sums, did not pay: 31 us stayed 31 us for two views, more views got slower.)
 template <bool CLAMP>
-__global__ void __launch_bounds__(32 * kAlphaPerBlock, 3) joseph_kernel(const RadonRow* __restrict__ table,
-                                                                         const RadonView* __restrict__ rv,
-                                                                         const float2* __restrict__ wimg,
+__global__ void __launch_bounds__(32 * kAlphaPerBlock, 3) joseph_kernel(const RadonRow* table,
+                                                                         const RadonView* rv,
+                                                                         const float2* wimg,
                                                                          JosephArgs g, float* __restrict__ out_f32,
                                                                          __nv_bfloat16* __restrict__ out_bf16) {
   wait_for_previous();
@@ -247,7 +247,7 @@ constexpr int kQuantBlock = 256 * 16;
 
 // Applies f to the values of this thread, f(index in the view, values).
 template <class F>
-__device__ __forceinline__ void quant_values(const float* __restrict__ p, size_t per_view, bool vec, F f) {
+__device__ __forceinline__ void quant_values(const float* p, size_t per_view, bool vec, F f) {
   const size_t i0 = (size_t)blockIdx.x * kQuantBlock;
   if (vec) {
     float4 x[4];
@@ -270,8 +270,7 @@ __device__ __forceinline__ void quant_values(const float* __restrict__ p, size_t
   }
 }
 
-__global__ void __launch_bounds__(256) absmax_kernel(const float* __restrict__ s32, size_t per_view, bool vec,
-                                                     RadonView* __restrict__ rv) {
+__global__ void __launch_bounds__(256) absmax_kernel(const float* s32, size_t per_view, bool vec, RadonView* rv) {
   wait_for_previous();
   struct {
     float m = 0.0f;
@@ -286,8 +285,7 @@ __global__ void __launch_bounds__(256) absmax_kernel(const float* __restrict__ s
   if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(&rv[blockIdx.y].max_bits, __float_as_uint(m));
 }
 
-__global__ void __launch_bounds__(256) quantize_f16_kernel(const float* __restrict__ s32, size_t per_view, bool vec,
-                                                           const RadonView* __restrict__ rv,
+__global__ void __launch_bounds__(256) quantize_f16_kernel(const float* s32, size_t per_view, bool vec, const RadonView* rv,
                                                            float* __restrict__ scales, __half* __restrict__ out) {
   wait_for_previous();
   const float m = __uint_as_float(rv[blockIdx.y].max_bits);

@@ -146,9 +146,8 @@ __device__ __forceinline__ void bulk_copy(unsigned dst, const void* src, unsigne
 constexpr int kTileX = 32, kTileY = 8;
 constexpr int kTilePitch = 33;
 
-__global__ void __launch_bounds__(256) weight_views_kernel(const float* __restrict__ images,
-                                                           const RadonView* __restrict__ rv, ViewsArgs g,
-                                                           float* __restrict__ planes) {
+__global__ void __launch_bounds__(256) weight_views_kernel(const float* __restrict__ images, const RadonView* rv,
+                                                           ViewsArgs g, float* __restrict__ planes) {
   wait_for_previous();
   __shared__ float tile[(kTileX + 1) * (kTileY + 1) * kTilePitch];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -381,9 +380,8 @@ __device__ __forceinline__ void fold(unsigned at, float4 (&acc)[kLines]) {
   tmem_stored();
 }
 
-__global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const RadonRow* __restrict__ table,
-                                                                     const RadonView* __restrict__ rv,
-                                                                     const float* __restrict__ planes, ViewsArgs g,
+__global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const RadonRow* table, const RadonView* rv,
+                                                                     const float* planes, ViewsArgs g,
                                                                      float* __restrict__ out_f32,
                                                                      __nv_bfloat16* __restrict__ out_bf16,
                                                                      int* __restrict__ status) {
@@ -407,7 +405,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) radon_views_kernel(const Radon
   const int m_end = cols ? g.r2 : ty >= t1 ? g.n_alpha : g.r1;
   const int steps = cols ? g.W : g.H, cells = cols ? g.H : g.W;
   const int pitch = cells + 1 + 2 * g.pad;
-  const float* __restrict__ plane =
+  const float* plane =
       planes + (cols ? g.cols0 : 0) + (size_t)blockIdx.z * steps * pitch * kGroup;
   const int blocks = g.A / kRows;  // of the alpha rows of one warp
   const int m_warp = m0 + (warp % blocks) * kRows;
