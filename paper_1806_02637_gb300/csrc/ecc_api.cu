@@ -194,12 +194,11 @@ int check_geometry_args(ecc_ctx* c, int n_views, const void* P, int W, int H, in
 // the weighted images of 13 groups of 32 views on the 768 x 768 grid of a 620 x 480 detector,
 // or of four on the 1024 x 1382 grid of a 976 x 976 one.
 constexpr size_t kViewsScratch = (size_t)1152 << 20;
-// Views per upload of the host-buffer call, and of its first, which nothing overlaps.  The line
-// sums of one group (1.85 ms on 620 x 480) take longer than the upload of the next 256 views
-// (1.5 ms at 205 GB/s), and each pass costs about 0.4 ms in weights and a last wave: 496 views
-// in passes of 32 and 256 take 24.75 ms, of 32 and 128 25.6, of 128 25.7, of 464 25.3, without
-// uploads 24.15.
-constexpr int kHostBatch = 256, kHostLead = 32;
+// Views of the host-buffer call's first upload, which nothing overlaps: one group.  Its line
+// sums (1.85 ms on 620 x 480) cover the upload of the next 128 views from 85 GB/s on (the rate
+// differs between boxes, 200 GB/s and about half of it), theirs that of the rest; each pass
+// costs about 0.4 ms in weights and a last wave.
+constexpr int kHostLead = 32;
 
 // Chooses the plan of a precompute and allocates its scratch.  In a context with a budget no
 // buffer of the many-view form is larger than the view-by-view form's on the same call, so
@@ -207,7 +206,7 @@ constexpr int kHostBatch = 256, kHostLead = 32;
 // only grow); less where the budget has less left.  Without a budget the form takes up to
 // kViewsScratch, and where the device has no such memory falls back to that.  n_scan: views of
 // the scan that these are part of.
-int ensure_precompute(ecc_ctx* c, int n_scan, int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
+int ensure_precompute(ecc_ctx* c, int n_scan, int n_views, int W, int H, int n_alpha, int n_s, int dtype,
                       ecc::RadonPlan* plan) {
   int rc;
   if ((rc = ensure(c, c->views, sizeof(ecc::ViewRec) * (size_t)n_views, "views")) != ECC_OK) return rc;
@@ -233,11 +232,11 @@ int ensure_precompute(ecc_ctx* c, int n_scan, int n_views, int W, int H, int n_a
     return rc == ECC_OK;
   };
   if (!c->budget) {
-    const ecc::RadonPlan p = ecc::radon_plan(n_scan, n_views, W, H, n_alpha, n_s, dtype, max_batch, large);
+    const ecc::RadonPlan p = ecc::radon_plan(n_scan, n_views, W, H, n_alpha, n_s, dtype, large);
     if (choose(p) || !p.views) return rc;
     drop_precompute(c);
   }
-  const ecc::RadonPlan p = ecc::radon_plan(n_scan, n_views, W, H, n_alpha, n_s, dtype, max_batch, small);
+  const ecc::RadonPlan p = ecc::radon_plan(n_scan, n_views, W, H, n_alpha, n_s, dtype, small);
   if (choose(p) || !p.views) return rc;
   if (!c->budget) drop_precompute(c);
   choose(by_view);
@@ -516,7 +515,7 @@ int ecc_precompute_radon_derivative_part(ecc_ctx* c, int n_scan_views, int n_vie
   if (dtype == ECC_F16 && !scales_out) return fail(c, ECC_EINVAL, "ECC_F16 needs scales_out");
   DeviceGuard g(c->device);
   ecc::RadonPlan plan;
-  if ((rc = ensure_precompute(c, n_scan_views, n_views, W, H, n_alpha, n_s, dtype, n_views, &plan)) != ECC_OK)
+  if ((rc = ensure_precompute(c, n_scan_views, n_views, W, H, n_alpha, n_s, dtype, &plan)) != ECC_OK)
     return rc;
   return run_precompute(c, n_views, P, images, W, H, n_alpha, n_s, dtype, sino_out, scales_out, plan,
                         (cudaStream_t)stream);
@@ -625,7 +624,7 @@ int ecc_scan_consistency_host(ecc_ctx* c, int n_views, const double* P_host, con
   // so that the upload of batch b + 1 overlaps the projection of batch b; pageable
   // memory (whose asynchronous copies block the host) is copied in one piece.
   ecc::RadonPlan plan;
-  if ((rc = ensure_precompute(c, n_views, n_views, W, H, n_alpha, n_s, ECC_F32, kHostBatch, &plan)) != ECC_OK) return rc;
+  if ((rc = ensure_precompute(c, n_views, n_views, W, H, n_alpha, n_s, ECC_F32, &plan)) != ECC_OK) return rc;
   if (plan.views) plan.lead = std::min(plan.batch, kHostLead);
   const int n_batches = plan.passes(n_views);
   cudaPointerAttributes pa;

@@ -166,10 +166,20 @@ struct RadonPlan {
   unsigned long long wait_ns = kWaitNs;
   bool views;          // many views at once
   int batch;           // views per pass over the scratch
-  int lead;            // views of the first pass
-  int passes(int n_views) const { return n_views <= lead ? 1 : 1 + (n_views - lead + batch - 1) / batch; }
-  int begin(int pass) const { return pass == 0 ? 0 : lead + (pass - 1) * batch; }
-  int count(int pass, int n_views) const { return std::min(pass == 0 ? lead : batch, n_views - begin(pass)); }
+  int lead;            // views of the first pass; each next one takes four times as many, up to batch
+  int passes(int n_views) const {
+    long long v = 0, size = lead;
+    int p = 0;
+    for (; v < n_views && size < batch; ++p, size = std::min<long long>(4 * size, batch)) v += size;
+    return p + (int)(v < n_views ? (n_views - v + batch - 1) / batch : 0);
+  }
+  int begin(int pass) const {
+    long long v = 0, size = lead;
+    int p = 0;
+    for (; p < pass && size < batch; ++p, size = std::min<long long>(4 * size, batch)) v += size;
+    return (int)std::min<long long>(v + (pass - p) * size, 0x7fffffff);
+  }
+  int count(int pass, int n_views) const { return std::min(begin(pass + 1), n_views) - begin(pass); }
   size_t wimg_bytes;   // weighted images
   size_t stage_bytes;  // FP32 staging of FP16 storage
   // the line table (copies of n_alpha rows) and the per-view weights after it
@@ -185,11 +195,9 @@ struct RadonPlan {
 struct RadonRoom {
   size_t wimg = SIZE_MAX, stage = SIZE_MAX, total = SIZE_MAX;
 };
-// The many-view form in the largest groups that fit the room, at most max_batch views (in
-// groups of 32) per pass.  Where none fits, or the scan does not qualify, the plan is the
-// view-by-view form's, which follows neither limit.
-RadonPlan radon_plan(int n_scan, int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
-                     const RadonRoom& room);
+// The many-view form in as many groups of 32 views at once as fit the room.  Where none fits,
+// or the scan does not qualify, the plan is the view-by-view form's, which follows no limit.
+RadonPlan radon_plan(int n_scan, int n_views, int W, int H, int n_alpha, int n_s, int dtype, const RadonRoom& room);
 RadonPlan radon_plan_by_view(int n_views, int W, int H, int n_alpha, int n_s, int dtype);
 
 // Many-view form, in groups of 32 views.

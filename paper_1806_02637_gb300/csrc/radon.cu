@@ -344,14 +344,13 @@ RadonPlan radon_plan_by_view(int n_views, int W, int H, int n_alpha, int n_s, in
   return p;
 }
 
-RadonPlan radon_plan(int n_scan, int n_views, int W, int H, int n_alpha, int n_s, int dtype, int max_batch,
+RadonPlan radon_plan(int n_scan, int n_views, int W, int H, int n_alpha, int n_s, int dtype,
                      const RadonRoom& room) {
   const int least = ViewsPlan::min_views(W, H, n_alpha, n_s);
   if (least > 0 && n_scan >= least) {
     for (int axes = 2; axes >= 1; --axes) {
       const size_t gb = ViewsPlan::group_bytes(axes, W, H, n_alpha, n_s);
       int groups = (int)std::min<size_t>((size_t)(n_views + 31) / 32, room.wimg / gb);
-      groups = std::min(groups, (max_batch + 31) / 32);
       auto batch = [&] { return std::min(n_views, groups * 32); };
       auto stage = [&] { return stage_bytes(n_alpha, n_s, dtype, batch()); };
       while (groups > 0 && (stage() > room.stage || gb * groups + stage() > room.total)) --groups;
@@ -405,7 +404,8 @@ cudaError_t launch_radon(int n_views, const float* images, int W, int H, int n_a
   const size_t per_view = (size_t)n_alpha * n_s;
   float2* wv = reinterpret_cast<float2*>(wimg);
   const bool behind = batch_ready == nullptr;  // behind an event a batch's first kernel is launched plainly
-  for (int pass = 0; pass < plan.passes(n_views); ++pass) {
+  const int passes = plan.passes(n_views);
+  for (int pass = 0; pass < passes; ++pass) {
     const int v0 = plan.begin(pass), nb = plan.count(pass, n_views);
     cudaError_t e;
     if (batch_ready && (e = cudaStreamWaitEvent(stream, batch_ready[pass], 0)) != cudaSuccess) return e;

@@ -102,7 +102,7 @@ Layout layout_of(const ecc_job& j) {
   const size_t wimg = align256(L.rtable + L.plan.table_bytes((int)n, j.n_alpha));
   ecc::RadonRoom room;
   room.total = o - wimg - 256;
-  L.plan = ecc::radon_plan((int)n, (int)n, j.W, j.H, j.n_alpha, j.n_s, j.dtype, (int)n, room);
+  L.plan = ecc::radon_plan((int)n, (int)n, j.W, j.H, j.n_alpha, j.n_s, j.dtype, room);
   if (L.plan.views) {
     L.wimg = wimg;
     L.stage = wimg + align256(L.plan.wimg_bytes);

@@ -11,7 +11,7 @@ torch = pytest.importorskip("torch")
 
 
 @pytest.mark.parametrize("n,W,Hh,n_alpha,n_s,kernel,passes", [
-    (300, 300, 260, 512, 400, "weight_views_kernel", 3),   # 32, 256 and 12 views
+    (300, 300, 260, 512, 400, "weight_views_kernel", 3),   # 32, 128 and 140 views
     (100, 620, 480, 90, 300, "weight_kernel", 3),          # lines too far apart for the form: 38, 38 and 24
 ])
 def test_uploads_in_passes(n, W, Hh, n_alpha, n_s, kernel, passes):
