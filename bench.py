@@ -772,11 +772,11 @@ def run_ours(args):
         flops = FLOPS_PER_TAP * taps * args.steps / n_dom
         achieved = flops / (ms_dom / n_dom / 1e3) / 1e12
         # DRAM bytes (read + write) of one launch, from ncu captures (joseph_kernel: 32 views, 183.3 MB +
-        # 58.3 MB; radon_views_kernel: 128 views, 400.7 MB + 276.1 MB), scaled to the views of an average
+        # 58.3 MB; radon_views_kernel: 128 views, 402.0 MB + 279.7 MB), scaled to the views of an average
         # launch of this step
         views_per_launch = cfg.n_views * args.steps / n_dom
         captured, per_view = ((32, (183.299840e6 + 58.299392e6) / 32) if dom == "joseph_kernel" else
-                              (128, (400.717056e6 + 276.057088e6) / 128))
+                              (128, (402.002432e6 + 279.659008e6) / 128))
         roof = {"kernel": dom, "bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": achieved / FP32_PEAK_TFLOPS, "traffic": per_view * views_per_launch,
                 "traffic_source": f"ncu dram__bytes_read.sum + dram__bytes_write.sum of a {captured}-view launch, "
@@ -792,7 +792,7 @@ def run_ours(args):
                                  "work": "8 B (one interpolation pair) per in-image tap"}
         else:
             # one walk along a line serves 32 views: no single limiter (ncu, 128 views)
-            roof["limits"] = {"issue": 0.67, "shared_memory_reads": 0.68, "fma_pipes": 0.54,
+            roof["limits"] = {"issue": 0.69, "shared_memory_reads": 0.65, "fma_pipes": 0.49,
                               "source": "ncu, 128 views of 620 x 480 on the 768 x 768 grid, of each peak"}
     else:
         bytes_per_launch = 32.0 * units * args.steps / n_dom

@@ -682,15 +682,15 @@ static Tiles tiles_of(int W, int H, int n_alpha, int n_s) {
   return t;
 }
 
-// A group takes as long as about 15 views of the view-by-view form where its CTAs fill the
-// GPU for some waves (one group against 15 and 16 views, in us: 1,701 against 1,644 and
-// 1,756 on 620 x 480, 6,030 against 6,349 and 6,790 on 976 x 976), and longer in proportion
-// where they do not: on 256 x 256 (102 CTAs a group) two groups take 412 against 389 for 39
-// views, on 300 x 260 (221 CTAs) one takes 479 against 440 for 20 and 486 against 546 for 25.
-// Where lines are closer together than a cell (more work per line, and windows with more
-// lines) it takes up to half as long again (97 views of 18 x 126, ds = 0.46: 139 against 93);
-// there from the second group on, whose last views may be few.  A rule on the sizes alone, at
-// which the many-view form was the faster one on ten grids: two waves of a GPU of 152 SMs.
+// A group takes as long as about 16 views of the view-by-view form where its CTAs fill the
+// GPU for some waves (one group of 16 views against 15 view by view, in us: 1,778 and 1,646 on
+// 620 x 480, 6,411 and 6,363 on 976 x 976), and longer in proportion where they do not
+// (300 x 260, 221 CTAs a group: 23 views 506, view by view 22 take 484; 256 x 256, 102 CTAs:
+// 48 and 47 views 434 and 484).  Where lines are closer together than a cell (windows with
+// more lines) it takes up to half as long again; there from the second group on, whose last
+// views may be few (168 views of 18 x 126, ds = 0.46: 188 and 188).  A rule on the sizes
+// alone, at which the two forms took about the same time on ten grids: two waves of a GPU of
+// 152 SMs.
 int ViewsPlan::min_views(int W, int H, int n_alpha, int n_s) {
   const Tiles t = tiles_of(W, H, n_alpha, n_s);
   if (t.A == 0) return 0;
